@@ -409,14 +409,16 @@ void adc_set_spin_limit(int64_t iterations);
 void adc_debug_set_stall_tile(int64_t tile);
 
 /*
- * Test hook: scan engine selection -- 0 automatic (range-partitioned for large
- * n, per-tile look-back otherwise), 1 per-tile look-back only, 2 range-
+ * Test hook: scan engine selection -- 0 automatic (streaming from 3 MB per
+ * input array on; without a streaming form range-partitioned for large n;
+ * per-tile look-back otherwise), 1 per-tile look-back only, 2 range-
  * partitioned wherever it applies, 3 range-partitioned with the range staged
  * in shared memory by bulk (TMA) copies, 4 per-tile look-back with each
  * block's tile staged in shared memory by bulk copies, 5 the range engine with
  * 16 bytes of each array per thread per tile, 6 the bulk-staged segment forms
  * of the q x q matrix scans (ADC_OP_MM3 / ADC_OP_MM5; also what 0 picks for
- * them, while 1 and 2 pick their register forms).  Other values restore 0.
+ * them, while 1 and 2 pick their register forms), 7 the streaming engine at
+ * every size where the operator has a streaming form.  Other values restore 0.
  * In the fault-injection hook
  * above, the "tile" of the range engines is a range.
  */

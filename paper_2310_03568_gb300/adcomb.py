@@ -282,7 +282,7 @@ def debug_force_hist_strategy(strategy):
 def debug_set_scan_engine(engine):
     """0 automatic, 1 per-tile look-back only, 2 range-partitioned wherever it applies, 3 TMA-staged
     ranges, 4 TMA-staged tiles, 5 ranges with 16 bytes per thread per tile, 6 the bulk-staged matrix
-    segment forms (see adc_debug_set_scan_engine)."""
+    segment forms, 7 the streaming engine at every size (see adc_debug_set_scan_engine)."""
     lib().adc_debug_set_scan_engine(int(engine))
 
 

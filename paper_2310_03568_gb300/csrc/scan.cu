@@ -15,6 +15,7 @@
 #include "internal.h"
 #include "scan_engine.cuh"
 #include "scan_mmq.cuh"
+#include "scan_stream.cuh"
 #include "scan_tma.cuh"
 #include "scan_staged.cuh"
 #include "tile_io.cuh"
@@ -107,15 +108,24 @@ template <typename E, int ITEMS, class Derived> struct PlainScan {
     __device__ void fetch_staged(const E *const (&sm)[1], int64_t lo, int64_t c0, int64_t n, Raw &r) const {
         load_chunk_sm(sm[0] + lo, c0, n, r.v, static_cast<const Derived *>(this)->identity());
     }
+    // streamed (scan_stream.cuh)
+    static constexpr int kWalk = 0;
+    __device__ E *dst() const { return y; }
+    __device__ bool accumulating() const { return false; }
+    __device__ E pad(int) const { return static_cast<const Derived *>(this)->identity(); }
+    __device__ State item(const E &v) const { return v; }
+    __device__ E out(const State &run, int64_t) const { return run; }
 };
 
 template <typename T, int ITEMS> struct FwdAdd : PlainScan<T, ITEMS, FwdAdd<T, ITEMS>> {
+    using Scalar = T;
     static constexpr bool kKeepPrefix = sizeof(T) == 8;  // fp64: the combine is the bound
     __device__ T identity() const { return T(0); }
     __device__ T combine(T a, T b) const { return a + b; }
 };
 
 template <typename T, int ITEMS> struct FwdMul : PlainScan<T, ITEMS, FwdMul<T, ITEMS>> {
+    using Scalar = T;
     static constexpr bool kKeepPrefix = sizeof(T) == 8;  // fp64: the combine is the bound
     __device__ T identity() const { return T(1); }
     __device__ T combine(T a, T b) const { return a * b; }
@@ -124,6 +134,7 @@ template <typename T, int ITEMS> struct FwdMul : PlainScan<T, ITEMS, FwdMul<T, I
 // min / max scans: the running extremum; the earlier operand wins ties (the
 // lifted operator of Fig. 5 with the lowest index first).
 template <typename T, int ITEMS, bool MAX> struct FwdSel : PlainScan<T, ITEMS, FwdSel<T, ITEMS, MAX>> {
+    using Scalar = T;
     static constexpr bool kKeepPrefix = sizeof(T) == 8;  // fp64: the combine is the bound
     __device__ T identity() const { return MAX ? -Num<T>::inf() : Num<T>::inf(); }
     __device__ T combine(T a, T b) const { return (MAX ? (b > a) : (b < a)) ? b : a; }
@@ -138,10 +149,15 @@ template <typename T, int ITEMS, bool MAX> struct FwdSel : PlainScan<T, ITEMS, F
         for (int k = 0; k < ITEMS; ++k) out[k] = x0 != x0 ? x0 : st[k];
         store_chunk(this->y, c0, n, out);
     }
+    __device__ T out(T run, int64_t) const {
+        const T x0 = __ldg(this->x);
+        return x0 != x0 ? x0 : run;
+    }
 };
 
 // linFnComp (Fig. 8): (b1,c1) . (b2,c2) = (b2 + c2*b1, c2*c1)
 template <typename T, int ITEMS> struct FwdLin : PlainScan<Pair<T>, ITEMS, FwdLin<T, ITEMS>> {
+    using Scalar = T;
     static constexpr bool kKeepPrefix = sizeof(T) == 8;  // fp64: the combine is the bound
     __device__ Pair<T> identity() const { return {T(0), T(1)}; }
     __device__ Pair<T> combine(const Pair<T> &a, const Pair<T> &b) const { return {b.b + b.c * a.b, b.c * a.c}; }
@@ -149,6 +165,7 @@ template <typename T, int ITEMS> struct FwdLin : PlainScan<Pair<T>, ITEMS, FwdLi
 
 // sumOfProd (Fig. 8): (p1,s1) . (p2,s2) = (p1 + p2 + s1*s2, s1 + s2)
 template <typename T, int ITEMS> struct FwdSop : PlainScan<Pair<T>, ITEMS, FwdSop<T, ITEMS>> {
+    using Scalar = T;
     static constexpr bool kKeepPrefix = sizeof(T) == 8;  // fp64: the combine is the bound
     __device__ Pair<T> identity() const { return {T(0), T(0)}; }
     __device__ Pair<T> combine(const Pair<T> &a, const Pair<T> &b) const {
@@ -157,6 +174,7 @@ template <typename T, int ITEMS> struct FwdSop : PlainScan<Pair<T>, ITEMS, FwdSo
 };
 
 template <typename T, int ITEMS> struct FwdMM2 : PlainScan<Mat2<T>, ITEMS, FwdMM2<T, ITEMS>> {
+    using Scalar = T;
     static constexpr bool kKeepPrefix = sizeof(T) == 8;  // fp64: the combine is the bound
     __device__ Mat2<T> identity() const { return mat_eye<T>(); }
     __device__ Mat2<T> combine(const Mat2<T> &a, const Mat2<T> &b) const { return mat_mul(a, b); }
@@ -181,6 +199,13 @@ template <typename T, int ITEMS> struct VjpAdd {
     __device__ void fetch_staged(const T *const (&sm)[1], int64_t lo, int64_t c0, int64_t n, Raw &r) const {
         load_chunk_sm(sm[0] + lo, c0, n, r.v, T(0));
     }
+    static constexpr int kWalk = 0;
+    using Scalar = T;
+    __device__ T *dst() const { return xbar; }
+    __device__ bool accumulating() const { return accumulate != 0; }
+    __device__ T pad(int) const { return T(0); }
+    __device__ T item(T v) const { return v; }
+    __device__ T out(T run, int64_t) const { return run; }
     __device__ void build(int64_t, int64_t, const Raw &r, T (&st)[ITEMS], Aux &) const {
 #pragma unroll
         for (int k = 0; k < ITEMS; ++k) st[k] = r.v[k];
@@ -234,6 +259,13 @@ template <typename T, int ITEMS> struct VjpMul {
         fetch_next_sm(sm[1], lo, c0, n, r.x, T(1));
         fetch_prev_sm(sm[2], lo, c0, n, r.y, T(1));
     }
+    static constexpr int kWalk = 1;
+    using Scalar = T;
+    __device__ Elem *dst() const { return xbar; }
+    __device__ bool accumulating() const { return accumulate != 0; }
+    __device__ T pad(int s) const { return s == 0 ? T(0) : T(1); }
+    __device__ State item(T yb, T xn) const { return {yb, xn}; }
+    __device__ T out(const State &run, T yp) const { return yp * run.v; }
     __device__ void build(int64_t c0, int64_t n, const Raw &r, State (&st)[ITEMS], Aux &aux) const {
 #pragma unroll
         for (int k = 0; k < ITEMS; ++k) {
@@ -282,6 +314,17 @@ template <typename T, int ITEMS, bool MAX> struct VjpSel {
     __device__ void fetch_staged(const T *const (&sm)[2], int64_t lo, int64_t c0, int64_t n, Raw &r) const {
         load_chunk_sm(sm[0] + lo, c0, n, r.yb.v, T(0));
         fetch_both_sm(sm[1], lo, c0, n, r.y, T(0));
+    }
+    static constexpr int kWalk = 2;
+    using Scalar = T;
+    __device__ Elem *dst() const { return xbar; }
+    __device__ bool accumulating() const { return accumulate != 0; }
+    __device__ T pad(int) const { return T(0); }
+    __device__ State item(T yb, T yi, T yn, int64_t i, int64_t n) const {
+        return {yb, (i + 1 < n && !same_value(yn, yi)) ? T(0) : T(1)};
+    }
+    __device__ T out(const State &run, T yi, T yp, int64_t i) const {
+        return ((i == 0 || !same_value(yi, yp)) ? T(1) : T(0)) * run.v;
     }
     __device__ void build(int64_t c0, int64_t n, const Raw &r, State (&st)[ITEMS], Aux &aux) const {
 #pragma unroll
@@ -336,6 +379,15 @@ template <typename T, int ITEMS> struct VjpLin {
         load_chunk_sm(sm[0] + lo, c0, n, r.yb.v, Pair<T>{T(0), T(0)});
         fetch_next_sm(sm[1], lo, c0, n, r.x, e);
         fetch_prev_sm(sm[2], lo, c0, n, r.y, e);
+    }
+    static constexpr int kWalk = 1;
+    using Scalar = T;
+    __device__ Elem *dst() const { return xbar; }
+    __device__ bool accumulating() const { return accumulate != 0; }
+    __device__ Pair<T> pad(int s) const { return {T(0), s == 0 ? T(0) : T(1)}; }
+    __device__ State item(const Pair<T> &yb, const Pair<T> &xn) const { return {yb.b, yb.c, xn.c}; }
+    __device__ Pair<T> out(const State &run, const Pair<T> &yp) const {
+        return {run.vb, run.vb * yp.b + run.vc * yp.c};
     }
     __device__ void build(int64_t c0, int64_t n, const Raw &r, State (&st)[ITEMS], Aux &aux) const {
 #pragma unroll
@@ -396,6 +448,13 @@ template <typename T, int ITEMS> struct VjpSop {
         fetch_next_sm(sm[1], lo, c0, n, r.x, z);
         fetch_prev_sm(sm[2], lo, c0, n, r.y, z);
     }
+    static constexpr int kWalk = 1;
+    using Scalar = T;
+    __device__ Elem *dst() const { return xbar; }
+    __device__ bool accumulating() const { return accumulate != 0; }
+    __device__ Pair<T> pad(int) const { return {T(0), T(0)}; }
+    __device__ State item(const Pair<T> &yb, const Pair<T> &xn) const { return {yb.b, yb.c, xn.c}; }
+    __device__ Pair<T> out(const State &run, const Pair<T> &yp) const { return {run.vp, yp.c * run.vp + run.vs}; }
     __device__ void build(int64_t c0, int64_t n, const Raw &r, State (&st)[ITEMS], Aux &aux) const {
 #pragma unroll
         for (int k = 0; k < ITEMS; ++k) {
@@ -444,6 +503,13 @@ template <typename T, int ITEMS> struct VjpMM2 {
         fetch_next_sm(sm[1], lo, c0, n, r.x, mat_eye<T>());
         fetch_prev_sm(sm[2], lo, c0, n, r.y, mat_eye<T>());
     }
+    static constexpr int kWalk = 1;
+    using Scalar = T;
+    __device__ Elem *dst() const { return xbar; }
+    __device__ bool accumulating() const { return accumulate != 0; }
+    __device__ Mat2<T> pad(int s) const { return s == 0 ? mat_zero<T>() : mat_eye<T>(); }
+    __device__ State item(const Mat2<T> &yb, const Mat2<T> &xn) const { return {yb, mat_t(xn)}; }
+    __device__ Mat2<T> out(const State &run, const Mat2<T> &yp) const { return mat_mul(mat_t(yp), run.v); }
     __device__ void build(int64_t c0, int64_t n, const Raw &r, State (&st)[ITEMS], Aux &aux) const {
 #pragma unroll
         for (int k = 0; k < ITEMS; ++k) {
@@ -741,6 +807,37 @@ template <class Op, int ITEMS, bool REVERSE>
 static adc_status launch(const Op &o, int64_t n, void *ws, cudaStream_t s) {
     return run_scan<Op, ITEMS, REVERSE>(o, n, ws, 0, static_cast<char *>(ws) + kWsHeader, s);
 }
+// The streaming engine's shape per operator (n = 1e8 fp32, n = 1e7 fp64; the
+// figures are this shape's against the next best one measured).  One input
+// array: 128-byte rows, 6 stages of 32 KB, fold and store by the same warps
+// (+ 0.138 / lin 0.284 ms forward; split 0.148 / 0.296).  The vjps of two and
+// three arrays: 64-byte rows, 4 stages of up to 48 KB; in fp32 the smem left is
+// short of the look-back's latency, and separate fold and store warps make up
+// for part of it (lin vjp 0.617 ms; same warps 0.721); in fp64 the second set of
+// warps only contends for the FP64 pipe (* vjp 0.149 ms; split 0.235).
+template <class Op> struct StreamPick {
+    static constexpr bool one = Op::kStreams == 1;
+    static constexpr bool f32 = sizeof(typename Op::Scalar) == 4;
+    static constexpr int kRow = one ? 128 : 64, kStages = one ? 6 : 4, kAhead = one || !f32 ? 2 : 1;
+    static constexpr bool kSplit = !one && f32;
+};
+// From 3 MB per input array on (about one 32 KB tile for every second SM) the
+// streaming engine is the faster one at every size measured: + n = 1e6 0.0139 ->
+// 0.0133 ms, 2e6 0.0214 -> 0.0157, 1e7 0.0352 -> 0.0235, 1e8 0.215 -> 0.138;
+// below, both are bound by their launches and the per-tile engine has the
+// smaller blocks.  A tuned range length asks for the range engine.
+constexpr int64_t kStreamMinBytes = 3 << 20;
+
+template <class Op, int ITEMS, bool REVERSE>
+static adc_status launch_auto(const Op &o, int64_t n, void *ws, cudaStream_t s) {
+    using P = StreamPick<Op>;
+    const bool stream = g_scan_engine == 7 || (g_scan_engine == 0 && g_scan_range_tiles == 0 &&
+                                               n * (int64_t)sizeof(typename Op::Elem) >= kStreamMinBytes);
+    if (stream && stream_ready<Op, 8, P::kRow, P::kStages, P::kAhead, P::kSplit, REVERSE>())
+        return run_scan_stream<Op, 8, P::kRow, P::kStages, P::kAhead, P::kSplit, REVERSE>(
+            o, n, ws, 0, static_cast<char *>(ws) + kWsHeader, ScanShape<Op, ITEMS>::region(n), s);
+    return launch<Op, ITEMS, REVERSE>(o, n, ws, s);
+}
 template <class Op, int ITEMS, bool REVERSE>
 static adc_status launch_staged(const Op &o, int64_t n, void *ws, cudaStream_t s) {
     if (g_scan_engine == 4) return run_scan_tma<Op, ITEMS, REVERSE>(o, n, ws, 0, static_cast<char *>(ws) + kWsHeader, s);
@@ -884,12 +981,12 @@ static adc_status scan_fwd_t(adc_op op, int64_t n, const void *x, void *y, void 
             FwdSel<T, I::scalar, true> o;
             o.x = static_cast<const T *>(x);
             o.y = static_cast<T *>(y);
-            return launch<decltype(o), I::scalar, false>(o, n, ws, s);
+            return launch_auto<decltype(o), I::scalar, false>(o, n, ws, s);
         }
         FwdSel<T, I::scalar, false> o;
         o.x = static_cast<const T *>(x);
         o.y = static_cast<T *>(y);
-        return launch<decltype(o), I::scalar, false>(o, n, ws, s);
+        return launch_auto<decltype(o), I::scalar, false>(o, n, ws, s);
     }
     if ((op == ADC_OP_MM3 || op == ADC_OP_MM5) && mmq_staged_ok()) {
         if (op == ADC_OP_MM3) return mmq_fwd_staged<T, 3>(n, x, y, ws, s);
@@ -947,31 +1044,34 @@ static adc_status scan_fwd_t(adc_op op, int64_t n, const void *x, void *y, void 
         FwdAdd<T, I::scalar> o;
         o.x = static_cast<const T *>(x);
         o.y = static_cast<T *>(y);
-        return launch<decltype(o), I::scalar, false>(o, n, ws, s);
+        return launch_auto<decltype(o), I::scalar, false>(o, n, ws, s);
     }
     case ADC_OP_MUL: {
         FwdMul<T, I::scalar> o;
         o.x = static_cast<const T *>(x);
         o.y = static_cast<T *>(y);
-        return launch<decltype(o), I::scalar, false>(o, n, ws, s);
+        return launch_auto<decltype(o), I::scalar, false>(o, n, ws, s);
     }
     case ADC_OP_LIN: {
         FwdLin<T, I::pair> o;
         o.x = static_cast<const Pair<T> *>(x);
         o.y = static_cast<Pair<T> *>(y);
-        return launch<decltype(o), I::pair, false>(o, n, ws, s);
+        return launch_auto<decltype(o), I::pair, false>(o, n, ws, s);
     }
     case ADC_OP_MM2: {
         FwdMM2<T, I::mat> o;
         o.x = static_cast<const Mat2<T> *>(x);
         o.y = static_cast<Mat2<T> *>(y);
+        // (an fp64 stage with its prefixes leaves too few of them; the 2x2 vjp's
+        // 8-word state makes the look-back the bound: 0.34 against 0.22 ms, n = 1e7)
+        if constexpr (sizeof(T) == 4) return launch_auto<decltype(o), I::mat, false>(o, n, ws, s);
         return launch<decltype(o), I::mat, false>(o, n, ws, s);
     }
     case ADC_OP_SOP: {
         FwdSop<T, I::pair> o;
         o.x = static_cast<const Pair<T> *>(x);
         o.y = static_cast<Pair<T> *>(y);
-        return launch<decltype(o), I::pair, false>(o, n, ws, s);
+        return launch_auto<decltype(o), I::pair, false>(o, n, ws, s);
     }
     default: return ADC_ERR_UNSUPPORTED;
     }
@@ -999,11 +1099,11 @@ static adc_status scan_vjp_t(adc_op op, int64_t n, const void *x, const void *y,
         if (op == ADC_OP_MAX) {
             VjpSel<T, I::vscalar, true> o{static_cast<const T *>(x), static_cast<const T *>(y),
                                           static_cast<const T *>(ybar), static_cast<T *>(xbar), acc};
-            return launch<decltype(o), I::vscalar, true>(o, n, ws, s);
+            return launch_auto<decltype(o), I::vscalar, true>(o, n, ws, s);
         }
         VjpSel<T, I::vscalar, false> o{static_cast<const T *>(x), static_cast<const T *>(y),
                                        static_cast<const T *>(ybar), static_cast<T *>(xbar), acc};
-        return launch<decltype(o), I::vscalar, true>(o, n, ws, s);
+        return launch_auto<decltype(o), I::vscalar, true>(o, n, ws, s);
     }
     if ((op == ADC_OP_MM3 || op == ADC_OP_MM5) && mmq_staged_ok()) {
         if (op == ADC_OP_MM3) return mmq_vjp_staged<T, 3>(n, x, y, ybar, xbar, acc, ws, s);
@@ -1056,17 +1156,17 @@ static adc_status scan_vjp_t(adc_op op, int64_t n, const void *x, const void *y,
     switch (op) {
     case ADC_OP_ADD: {
         VjpAdd<T, I::scalar> o{static_cast<const T *>(ybar), static_cast<T *>(xbar), acc};
-        return launch<decltype(o), I::scalar, true>(o, n, ws, s);
+        return launch_auto<decltype(o), I::scalar, true>(o, n, ws, s);
     }
     case ADC_OP_MUL: {
         VjpMul<T, I::vscalar> o{static_cast<const T *>(x), static_cast<const T *>(y), static_cast<const T *>(ybar),
                                 static_cast<T *>(xbar), acc};
-        return launch<decltype(o), I::vscalar, true>(o, n, ws, s);
+        return launch_auto<decltype(o), I::vscalar, true>(o, n, ws, s);
     }
     case ADC_OP_LIN: {
         VjpLin<T, I::vpair> o{static_cast<const Pair<T> *>(x), static_cast<const Pair<T> *>(y),
                               static_cast<const Pair<T> *>(ybar), static_cast<Pair<T> *>(xbar), acc};
-        return launch<decltype(o), I::vpair, true>(o, n, ws, s);
+        return launch_auto<decltype(o), I::vpair, true>(o, n, ws, s);
     }
     case ADC_OP_MM2: {
         VjpMM2<T, I::vmat> o{static_cast<const Mat2<T> *>(x), static_cast<const Mat2<T> *>(y),
@@ -1076,7 +1176,7 @@ static adc_status scan_vjp_t(adc_op op, int64_t n, const void *x, const void *y,
     case ADC_OP_SOP: {
         VjpSop<T, I::vpair> o{static_cast<const Pair<T> *>(x), static_cast<const Pair<T> *>(y),
                               static_cast<const Pair<T> *>(ybar), static_cast<Pair<T> *>(xbar), acc};
-        return launch<decltype(o), I::vpair, true>(o, n, ws, s);
+        return launch_auto<decltype(o), I::vpair, true>(o, n, ws, s);
     }
     default: return ADC_ERR_UNSUPPORTED;
     }

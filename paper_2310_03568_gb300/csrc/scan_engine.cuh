@@ -703,7 +703,8 @@ template <class Op> constexpr int range_tiles_hint(long) { return 0; }
 template <class Op> constexpr auto range_tiles_hint(int) -> decltype(Op::kRangeTiles, int()) { return Op::kRangeTiles; }
 
 // Engine selection for tests and measurements: 0 automatic, 1 per-tile
-// look-back only, 2 range-partitioned where it applies.
+// look-back only, 2 range-partitioned where it applies, 7 streaming where it
+// applies (see adc_debug_set_scan_engine for the others).
 extern int g_scan_engine;
 extern int g_scan_range_tiles;
 
@@ -745,7 +746,7 @@ adc_status run_scan(const Op &op, int64_t n, void *ws, int slot, void *region, c
     if (rt > 0) R = (T + rt - 1) / rt;
     if (R > T) R = T;
     const bool ranges = T <= (int64_t)range_max_tiles<typename Op::State>() * R &&
-                        (g_scan_engine == 2 || g_scan_engine == 5 || (g_scan_engine == 0 && T >= 4 * G));
+                        (g_scan_engine == 2 || g_scan_engine == 5 || ((g_scan_engine == 0 || g_scan_engine == 7) && T >= 4 * G));
     if (ranges) {
         k_scan_ranges<Op, kScanThreads, ITEMS, REVERSE><<<(unsigned)R, kScanThreads, 0, s>>>(
             op, n, T, reinterpret_cast<unsigned long long *>(w + L.agg_off),
