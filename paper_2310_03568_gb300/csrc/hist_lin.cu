@@ -7,26 +7,31 @@
 //      run of 32 * R consecutive elements, R rounds of 32): every warp walks
 //      its run in index order and folds each element into its bin's entry of
 //      a warp-private table in shared memory.  Within a round, lanes holding
-//      the same bin (__match_any_sync peers) update one after another in lane
-//      order, so every bin's entry is the ordered fold of the run's values;
-//      the block then composes the warp tables per bin in warp order ->
-//      P[bin][chunk] (identity where the bin is absent);
-//   2. one block per bin composes its row of P in chunk order: the exclusive
-//      prefix L[bin][c] = hist0 . P[bin][0..c-1], the exclusive suffix
-//      R[bin][c] = P[bin][c+1..], hist = L . P at the last chunk and the bin
-//      total A = P[bin][0] . R[bin][0] (for hist0bar);
+//      the same bin update one after another in lane order, so every bin's
+//      entry is the ordered fold of the run's values; the block then composes
+//      the warp tables per bin in warp order -> P[chunk][bin] (identity where
+//      the bin is absent);
+//   2. per bin, its column of P in chunk order: the exclusive prefix
+//      L[c][bin] = hist0 . P[0..c-1][bin], the c's product of the exclusive
+//      suffix Rc[c][bin], hist and the bin total A (for hist0bar);
 //   3. vjp, per chunk: the forward walk again, keeping each element's
-//      exclusive prefix p_i within its warp run, and a backward walk keeping
-//      the product s_i of the c's after it; per bin and warp the block forms
-//      what lies before the run (L . earlier runs) and the product of the c's
-//      after it (later runs, R), and every element gets
+//      exclusive prefix p_i within its warp run, and a backward walk (the
+//      forward one's lane ranks, reversed) keeping the product s_i of the c's
+//      after it; per bin and warp the block forms what lies before the run
+//      (L . earlier runs) and the product of the c's after it (later runs,
+//      Rc), and every element gets
 //      vbar_i = d(l_i . v_i . r_i)/dv_i ^T histbar[k_i] with l_i = before . p_i
 //      and r_i.c = s_i * after.c.
 // Within every bin the values meet in index order, as the sequential
 // definition requires; only the bracketing differs (associativity).
 // Traffic: the forward reads keys and values once (12 B per fp32 element) and
-// moves the [m][chunks] matrices (P, L, R: 8 B per bin and chunk each); the
-// vjp reads keys, values, L and R and writes the adjoints once.
+// moves the [chunks][m] matrices (P and L 8 B, Rc 4 B per bin and chunk); the
+// vjp reads keys, values, L and Rc and writes the adjoints once.  Bound by the
+// latency of the walks' shared-memory steps, at 16 to 24 warps per SM (the
+// tables fill the shared memory).  n = 1e7, m = 1000, fp32: fold 0.074 -> 0.049
+// ms (ranks found by ballots a round ahead instead of a match in the update's
+// way), columns 0.037 -> 0.029 ms and vjp 0.189 -> 0.118 ms (ranks reused
+// backwards, chunk-major matrices).
 #include "common.cuh"
 #include "hist_common.cuh"
 #include "internal.h"
@@ -82,35 +87,58 @@ __device__ __forceinline__ void load_run(const int32_t *__restrict__ keys, const
     }
 }
 
-// One round of a warp walk: upd() runs for every lane with an in-range key,
-// in lane order among lanes that share a key (REV: descending lane order),
-// lanes with different keys at once.  Every such lane first writes its lane
-// number to its key's byte in `tag` (one byte per bin and warp): when each
-// reads its own number back, no two lanes share a key and all update in one
-// step; otherwise __match_any_sync groups the lanes and the groups advance
-// one rank per step.  Warp-wide: all lanes call it.
-template <bool REV, class F>
-__device__ __forceinline__ void ordered_round(int32_t key, bool ok, uint8_t *tag, F &&upd) {
+// Which lanes of a round share a bin, found one round ahead of the walk so that
+// the table update of one round and the search of the next overlap.  Every
+// lane with an in-range key writes its lane number to its key's byte in `tag`
+// (one byte per bin and warp); the lanes that do not read their own number
+// back share a bin with another lane.  Few of them (the usual case: about two
+// rounds in five at m = 1000 have one pair): each such key is broadcast and
+// balloted; many: __match_any_sync, whose cost does not grow with them but is
+// several times one ballot's.  Warp-wide: all lanes call tag_write / ranks.
+struct LRank {
+    uint8_t rank, cnt;  // the lane's place among the lanes with its bin (lane order), and their number
+};
+__device__ __forceinline__ void tag_write(int32_t key, bool ok, uint8_t *tag) {
+    if (ok) tag[key] = (uint8_t)(threadIdx.x & 31);
+}
+// After a __syncwarp() that follows tag_write(); true if two lanes share a bin.
+__device__ __forceinline__ bool ranks(int32_t key, bool ok, const uint8_t *tag, LRank &r) {
     const int lane = threadIdx.x & 31;
-    if (ok) tag[key] = (uint8_t)lane;
-    __syncwarp();
-    const bool alone = !ok || tag[key] == (uint8_t)lane;
-    if (__all_sync(0xffffffffu, alone)) {
+    unsigned lost = __ballot_sync(0xffffffffu, ok && tag[key] != (uint8_t)lane);
+    r = {0, 1};
+    if (lost == 0u) return false;
+    unsigned peers = 1u << lane;
+    if (__popc(lost) <= 4) {
+        while (lost) {
+            const int32_t k = __shfl_sync(0xffffffffu, key, __ffs(lost) - 1);
+            const unsigned same = __ballot_sync(0xffffffffu, ok && key == k);
+            if (ok && key == k) peers = same;
+            lost &= ~same;
+        }
+    } else {
+        peers = __match_any_sync(0xffffffffu, ok ? key : -1);
+        if (!ok) peers = 1u << lane;
+    }
+    r.rank = (uint8_t)__popc(peers & ((1u << lane) - 1u));
+    r.cnt = (uint8_t)__popc(peers);
+    return true;
+}
+// One round's updates: upd() runs for every lane with an in-range key, at once
+// when no two share a bin, else in rank order.
+template <class F>
+__device__ __forceinline__ void ranked_update(bool shared, bool ok, int rank, F &&upd) {
+    if (!shared) {
         if (ok) upd();
     } else {
-        const unsigned peers = __match_any_sync(0xffffffffu, ok ? key : -1);
-        const unsigned ahead = REV ? (peers & ~((2u << lane) - 1u)) : (peers & ((1u << lane) - 1u));
-        const int rank = __popc(ahead);
         for (int q = 0; __any_sync(0xffffffffu, ok && rank >= q); ++q) {
             if (ok && rank == q) upd();
             __syncwarp();
         }
     }
-    __syncwarp();
 }
 
 // ------------------------------------------------------------ chunk fold --
-// P[bin * nc + chunk] = ordered fold of the chunk's values of that bin.
+// P[chunk * m + bin] = ordered fold of the chunk's values of that bin.
 template <typename T>
 __global__ void __launch_bounds__(kLThreads)
 k_linh_fold(const int32_t *__restrict__ keys, const Pair<T> *__restrict__ vals, const int64_t n, const int m,
@@ -128,140 +156,105 @@ k_linh_fold(const int32_t *__restrict__ keys, const Pair<T> *__restrict__ vals, 
     load_run<T, C::kRounds>(keys, vals, c * C::kSize + (int64_t)warp * C::kRun, n, m, k, v);
     for (int j = lane; j < m; j += kWarp) tab[j] = lf_id<T>();
     __syncwarp();
+    LRank rk;
+    tag_write(k[0], in_range(k[0], m), tag);
+    __syncwarp();
+    bool shared = ranks(k[0], in_range(k[0], m), tag, rk);
 #pragma unroll
     for (int r = 0; r < C::kRounds; ++r) {
         const int32_t key = k[r];
         const Pair<T> x = v[r];
-        ordered_round<false>(key, in_range(key, m), tag, [&] { tab[key] = lf(tab[key], x); });
+        const int nx = r + 1 < C::kRounds ? r + 1 : r;
+        if (r + 1 < C::kRounds) tag_write(k[nx], in_range(k[nx], m), tag);
+        ranked_update(shared, in_range(key, m), rk.rank, [&] { tab[key] = lf(tab[key], x); });
+        __syncwarp();
+        if (r + 1 < C::kRounds) shared = ranks(k[nx], in_range(k[nx], m), tag, rk);
     }
     __syncthreads();
     for (int j = tid; j < m; j += kLThreads) {
         Pair<T> acc = s_tab[j];
 #pragma unroll
         for (int w = 1; w < kLWarps; ++w) acc = lf(acc, s_tab[(size_t)w * m + j]);
-        P[(int64_t)j * nc + c] = acc;
+        P[c * m + j] = acc;
     }
 }
 
-// ------------------------------------------------------------- bin rows --
-// Block-wide exclusive scan of one state per thread in thread order (REV:
-// reverse thread order) for linFnComp; two __syncthreads().
-template <typename T, bool REV>
-__device__ __forceinline__ Pair<T> lblock_excl(Pair<T> a, Pair<T> *s_w) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int vl = REV ? (kWarp - 1 - lane) : lane;
-    const int vw = REV ? (kLWarps - 1 - warp) : warp;
-    // REV: a forward scan over mirrored lanes and warps with the operands
-    // swapped (later elements come first in logical order)
-#pragma unroll
-    for (int o = 1; o < kWarp; o <<= 1) {
-        const Pair<T> up = REV ? shfl_down(a, o) : shfl_up(a, o);
-        if (vl >= o) a = REV ? lf(a, up) : lf(up, a);
-    }
-    if (vl == kWarp - 1) s_w[vw] = a;
-    Pair<T> ex = REV ? shfl_down(a, 1) : shfl_up(a, 1);
-    if (vl == 0) ex = lf_id<T>();
-    __syncthreads();
-    Pair<T> before = lf_id<T>();
-#pragma unroll
-    for (int w = 0; w < kLWarps; ++w)
-        if (w < vw) before = REV ? lf(s_w[w], before) : lf(before, s_w[w]);
-    __syncthreads();
-    return REV ? lf(ex, before) : lf(before, ex);
-}
-
-// One block per bin j: L[j][c], R[j][c], hist[j], A[j] from the row P[j][.].
-// The row goes through shared memory in segments of RI entries per thread
-// (loads and stores coalesced); within a segment thread t composes its RI
-// consecutive entries and a block scan gives what lies before (L) or after
-// (R) them.  A row that fits one segment is loaded once: the reverse pass
-// reuses each thread's entries from registers (fp32 takes 16 entries per
-// thread, so rows of up to 4096 chunks, n <= 16.7M, are one segment).
-template <typename T> constexpr int row_items() { return sizeof(T) == 4 ? 16 : 8; }
+// ---------------------------------------------------------- bin columns --
+// L[c][j] (what lies before chunk c in bin j: hist0 . P[0..c-1][j]), Rc[c][j]
+// (the product of the c's after it; the vjp needs no more of the suffix),
+// hist[j] and the bin total A[j], from the columns P[.][j].  The matrices are
+// chunk-major, so that the chunk kernels read and write them in order
+// (bin-major, each of a chunk's 8-byte cells was a sector of its own); a block
+// takes kColBins bins -- 64 contiguous bytes of a row -- and cuts their columns
+// into kColSegs segments, one thread each: fold the segment, combine the
+// segments through shared memory, walk it again forwards for L and backwards
+// for Rc (both walks read from L2).
+constexpr int kColBins = 8;
+constexpr int kColSegs = kLThreads / kColBins;
 
 template <typename T>
 __global__ void __launch_bounds__(kLThreads)
-k_linh_rows(const Pair<T> *__restrict__ P, const Pair<T> *__restrict__ h0, const int64_t nc,
-            Pair<T> *__restrict__ L, Pair<T> *__restrict__ R, Pair<T> *__restrict__ hist, Pair<T> *__restrict__ A) {
-    constexpr int RI = row_items<T>();
-    constexpr int SEG = kLThreads * RI;
-    __shared__ Pair<T> s_seg[SEG];
-    __shared__ Pair<T> s_w[kLWarps];
-    __shared__ Pair<T> s_tot;
-    const int tid = threadIdx.x;
-    const int64_t j = blockIdx.x;
-    const Pair<T> *row = P + j * nc;
-    const bool one = nc <= SEG;  // the whole row in one segment
-    Pair<T> v[RI], agg = lf_id<T>();
-    // forward: L = hist0 . the entries before
-    Pair<T> carry = h0 ? h0[j] : lf_id<T>();
-    for (int64_t s0 = 0; s0 < nc; s0 += SEG) {
-        const int len = (int)((nc - s0) < SEG ? (nc - s0) : SEG);
-        for (int e = tid; e < len; e += kLThreads) s_seg[e] = row[s0 + e];
-        __syncthreads();
-        agg = lf_id<T>();
+k_linh_cols(const Pair<T> *__restrict__ P, const Pair<T> *__restrict__ h0, const int64_t nc, const int64_t m,
+            Pair<T> *__restrict__ L, T *__restrict__ Rc, Pair<T> *__restrict__ hist, Pair<T> *__restrict__ A) {
+    constexpr int U = 8;  // loads in flight
+    __shared__ Pair<T> s_fold[kColSegs][kColBins];
+    const int b = threadIdx.x % kColBins, sg = threadIdx.x / kColBins;
+    const int64_t j = (int64_t)blockIdx.x * kColBins + b;
+    const bool live = j < m;
+    const int64_t per = (nc + kColSegs - 1) / kColSegs;
+    const int64_t c0 = sg * per < nc ? sg * per : nc, c1 = c0 + per < nc ? c0 + per : nc;
+    const Pair<T> *col = P + j;
+    Pair<T> f = lf_id<T>();
+    if (live)
+        for (int64_t c = c0; c < c1; c += U) {
+            Pair<T> x[U];
 #pragma unroll
-        for (int k = 0; k < RI; ++k) {
-            const int idx = tid * RI + k;
-            v[k] = idx < len ? s_seg[idx] : lf_id<T>();
-            agg = lf(agg, v[k]);
-        }
-        const Pair<T> ex = lblock_excl<T, false>(agg, s_w);
-        if (tid == kLThreads - 1) s_tot = lf(ex, agg);
-        Pair<T> run = lf(carry, ex);
+            for (int u = 0; u < U; ++u) x[u] = c + u < c1 ? col[(c + u) * m] : lf_id<T>();
 #pragma unroll
-        for (int k = 0; k < RI; ++k) {
-            const int idx = tid * RI + k;
-            if (idx < len) {
-                s_seg[idx] = run;
-                run = lf(run, v[k]);
-            }
+            for (int u = 0; u < U; ++u) f = lf(f, x[u]);
         }
-        __syncthreads();
-        for (int e = tid; e < len; e += kLThreads) L[j * nc + s0 + e] = s_seg[e];
-        carry = lf(carry, s_tot);
-        __syncthreads();
+    s_fold[sg][b] = f;
+    __syncthreads();
+    if (!live) return;
+    Pair<T> before = lf_id<T>();
+    for (int q = 0; q < sg; ++q) before = lf(before, s_fold[q][b]);
+    T after = T(1);
+    for (int q = kColSegs - 1; q > sg; --q) after = s_fold[q][b].c * after;
+    if (sg == kColSegs - 1) {
+        const Pair<T> all = lf(before, f);
+        A[j] = all;
+        hist[j] = h0 ? lf(h0[j], all) : all;
     }
-    if (tid == 0) hist[j] = carry;
-    // reverse: R = the entries after, from the last segment down
-    Pair<T> rcarry = lf_id<T>();
-    for (int64_t s0 = (nc - 1) / SEG * SEG; s0 >= 0; s0 -= SEG) {
-        const int len = (int)((nc - s0) < SEG ? (nc - s0) : SEG);
-        if (!one) {  // a single segment's entries are still in v
-            for (int e = tid; e < len; e += kLThreads) s_seg[e] = row[s0 + e];
-            __syncthreads();
-            agg = lf_id<T>();
+    Pair<T> run = h0 ? lf(h0[j], before) : before;
+    for (int64_t c = c0; c < c1; c += U) {
+        Pair<T> x[U];
 #pragma unroll
-            for (int k = 0; k < RI; ++k) {
-                const int idx = tid * RI + k;
-                v[k] = idx < len ? s_seg[idx] : lf_id<T>();
-                agg = lf(agg, v[k]);
-            }
-        }
-        const Pair<T> rex = lblock_excl<T, true>(agg, s_w);  // the later threads' entries
-        if (tid == 0) s_tot = lf(agg, rex);
-        Pair<T> rrun = lf(rex, rcarry);
+        for (int u = 0; u < U; ++u) x[u] = c + u < c1 ? col[(c + u) * m] : lf_id<T>();
 #pragma unroll
-        for (int k = RI - 1; k >= 0; --k) {
-            const int idx = tid * RI + k;
-            if (idx < len) {
-                s_seg[idx] = rrun;
-                rrun = lf(v[k], rrun);
+        for (int u = 0; u < U; ++u)
+            if (c + u < c1) {
+                L[(c + u) * m + j] = run;
+                run = lf(run, x[u]);
             }
-        }
-        __syncthreads();
-        for (int e = tid; e < len; e += kLThreads) R[j * nc + s0 + e] = s_seg[e];
-        rcarry = lf(s_tot, rcarry);
-        __syncthreads();
     }
-    if (tid == 0) A[j] = rcarry;  // P[j][0] . R[j][0]: the bin's whole fold
+    for (int64_t c = c1; c > c0; c -= U) {
+        T x[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) x[u] = c - 1 - u >= c0 ? col[(c - 1 - u) * m].c : T(1);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (c - 1 - u >= c0) {
+                Rc[(c - 1 - u) * m + j] = after;
+                after = x[u] * after;
+            }
+    }
 }
 
 // ------------------------------------------------------------------- vjp --
 template <typename T>
 __global__ void __launch_bounds__(kLThreads, 2)
 k_linh_vjp(const int32_t *__restrict__ keys, const Pair<T> *__restrict__ vals, const int64_t n, const int m,
-           const int64_t nc, const Pair<T> *__restrict__ L, const Pair<T> *__restrict__ R,
+           const int64_t nc, const Pair<T> *__restrict__ L, const T *__restrict__ Rc,
            const Pair<T> *__restrict__ hb, Pair<T> *__restrict__ vbar, const int accumulate) {
     using C = LChunk<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -284,18 +277,28 @@ k_linh_vjp(const int32_t *__restrict__ keys, const Pair<T> *__restrict__ vals, c
     }
     for (int j = tid; j < m; j += kLThreads) s_g[j] = hb[j];
     __syncwarp();
-    // forward walk: p_i = the run's fold of i's bin before i
+    // forward walk: p_i = the run's fold of i's bin before i; the ranks are kept
+    // for the backward walk, where the order is reversed
     Pair<T> p[C::kRounds];
+    LRank rk[C::kRounds];
+    unsigned shared = 0;  // bit r: lanes of round r share a bin (uniform)
+    tag_write(k[0], in_range(k[0], m), tag);
+    __syncwarp();
+    if (ranks(k[0], in_range(k[0], m), tag, rk[0])) shared |= 1u;
 #pragma unroll
     for (int r = 0; r < C::kRounds; ++r) {
         const int32_t key = k[r];
         const Pair<T> x = v[r];
+        const int nx = r + 1 < C::kRounds ? r + 1 : r;
+        if (r + 1 < C::kRounds) tag_write(k[nx], in_range(k[nx], m), tag);
         Pair<T> pr = lf_id<T>();
-        ordered_round<false>(key, in_range(key, m), tag, [&] {
+        ranked_update((shared >> r) & 1u, in_range(key, m), rk[r].rank, [&] {
             pr = tab[key];
             tab[key] = lf(pr, x);
         });
         p[r] = pr;
+        __syncwarp();
+        if (r + 1 < C::kRounds && ranks(k[nx], in_range(k[nx], m), tag, rk[nx])) shared |= 1u << nx;
     }
     // backward walk: s_i = product of the c's of i's bin after i in the run
     T sv[C::kRounds];
@@ -304,18 +307,19 @@ k_linh_vjp(const int32_t *__restrict__ keys, const Pair<T> *__restrict__ vals, c
         const int32_t key = k[r];
         const T xc = v[r].c;
         T sr = T(1);
-        ordered_round<true>(key, in_range(key, m), tag, [&] {
+        ranked_update((shared >> r) & 1u, in_range(key, m), rk[r].cnt - 1 - rk[r].rank, [&] {
             sr = qt[key];
             qt[key] = xc * sr;
         });
         sv[r] = sr;
+        __syncwarp();
     }
     __syncthreads();
     // per bin and warp run: u = <L . earlier runs, g> and the product of the
     // c's after the run (later runs, then R)
     for (int j = tid; j < m; j += kLThreads) {
         const Pair<T> g = s_g[j];
-        Pair<T> before = L[(int64_t)j * nc + c];
+        Pair<T> before = L[c * m + j];
         T fc[kLWarps], u[kLWarps];
 #pragma unroll
         for (int w = 0; w < kLWarps; ++w) {
@@ -324,7 +328,7 @@ k_linh_vjp(const int32_t *__restrict__ keys, const Pair<T> *__restrict__ vals, c
             fc[w] = f.c;
             before = lf(before, f);
         }
-        T after = R[(int64_t)j * nc + c].c;
+        T after = Rc[c * m + j];
 #pragma unroll
         for (int w = kLWarps - 1; w >= 0; --w) {
             s_tab[(size_t)w * m + j] = Pair<T>{u[w], after};
@@ -413,9 +417,9 @@ static adc_status linh_fwd_t(int64_t n, int64_t m, const int32_t *keys, const Pa
     if (cudaFuncSetAttribute(k_linh_fold<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return ADC_ERR_CUDA;
     k_linh_fold<T><<<(unsigned)nc, kLThreads, smem, s>>>(keys, vals, n, (int)m, nc, P);
-    k_linh_rows<T><<<(unsigned)m, kLThreads, 0, s>>>(P, h0, nc, reinterpret_cast<Pair<T> *>(sv + Lo.L),
-                                                     reinterpret_cast<Pair<T> *>(sv + Lo.R), hist,
-                                                     reinterpret_cast<Pair<T> *>(sv + Lo.A));
+    k_linh_cols<T><<<(unsigned)((m + kColBins - 1) / kColBins), kLThreads, 0, s>>>(
+        P, h0, nc, m, reinterpret_cast<Pair<T> *>(sv + Lo.L), reinterpret_cast<T *>(sv + Lo.R), hist,
+        reinterpret_cast<Pair<T> *>(sv + Lo.A));
     return check_launch();
 }
 
@@ -426,7 +430,7 @@ static adc_status linh_vjp_t(int64_t n, int64_t m, const int32_t *keys, const Pa
     const int64_t nc = num_chunks<T>(n);
     const char *sv = static_cast<const char *>(saved);
     const Pair<T> *L = reinterpret_cast<const Pair<T> *>(sv + Lo.L);
-    const Pair<T> *R = reinterpret_cast<const Pair<T> *>(sv + Lo.R);
+    const T *R = reinterpret_cast<const T *>(sv + Lo.R);
     const Pair<T> *A = reinterpret_cast<const Pair<T> *>(sv + Lo.A);
     if (n > 0) {
         const size_t smem = vjp_smem<T>(m);
