@@ -38,7 +38,7 @@ constexpr int kPartChunk = kPartThreads * kPartItems;  // 8192 elements
 constexpr int kPartMaxBuckets = 2048;
 constexpr int kPartTableThreads = 1024;
 constexpr size_t kPartTableBudget = 200 * 1024;  // one table block per SM
-constexpr int kPartSlot = 20;                    // workspace counter slot of the count scan
+constexpr int kPartSlot = 20;                    // workspace counter slot of the count's ticket
 
 // k / W for in-range keys by a float reciprocal and one correction step: the
 // quotients stay below 2^11, so the float estimate is off by at most one.
@@ -130,7 +130,8 @@ template <bool MAX> struct PartSel {
         reinterpret_cast<V *>(sm)[t] = Pack<MAX>::kEmpty;
     }
     // Few values per bin at the sizes this strategy serves: most updates win,
-    // so the atomic is issued without a read filter.
+    // so the atomic is issued without a read filter (with one the table pass at
+    // m = 1e7, n = 5e7 took 0.139 instead of 0.117 ms).
     template <int U>
     static __device__ __forceinline__ void update(unsigned char *sm, int, const int32_t (&u)[U], const V (&v)[U],
                                                   const bool (&use)[U], unsigned *) {
@@ -236,39 +237,88 @@ __device__ __forceinline__ void load_group(const int32_t *__restrict__ keys, con
     }
 }
 
-// 1. counts[b * nchunks + chunk] = elements of the chunk in bucket b; row B is
-// a zero row so that the scanned matrix also gives every bucket's end.
+// 1. Elements per bucket (persistent blocks, one shared-memory counter per
+// bucket); the last block to finish turns them into where every bucket's
+// elements go: start[b] (start[B] = their number) and the cursors that the
+// scatter's chunks advance.
 __global__ void __launch_bounds__(kPartThreads)
 k_part_count(const int32_t *__restrict__ keys, const int64_t n, const int64_t m, const BucketDiv bdiv, const int B,
-             const int64_t nchunks, int32_t *__restrict__ counts) {
+             int32_t *__restrict__ totals, int32_t *__restrict__ start, int32_t *__restrict__ cursor,
+             unsigned *__restrict__ ticket) {
+    constexpr int NW = kPartThreads / kWarp;
+    constexpr int PER = kPartMaxBuckets / kPartThreads;
     extern __shared__ int32_t s_cnt[];
-    for (int b = threadIdx.x; b < B; b += kPartThreads) s_cnt[b] = 0;
+    __shared__ int32_t s_part[NW];
+    __shared__ bool s_last;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int b = tid; b < B; b += kPartThreads) s_cnt[b] = 0;
     __syncthreads();
-    const int64_t c0 = (int64_t)blockIdx.x * kPartChunk;
+    constexpr int U = 4;
+    const auto add = [&](int32_t k) {
+        if (in_range(k, m)) atomicAdd(&s_cnt[bdiv((uint32_t)k)], 1);
+    };
+    const int64_t quads = n / 4, stride = (int64_t)gridDim.x * kPartThreads;
+    const int4 *k4 = reinterpret_cast<const int4 *>(keys);
+    for (int64_t q0 = (int64_t)blockIdx.x * kPartThreads + tid; q0 < quads; q0 += U * stride) {
+        int4 k[U];
 #pragma unroll
-    for (int r = 0; r < kPartItems / 4; ++r) {
-        int32_t kk[4];
-        float unused[4];
-        load_group<float>(keys, nullptr, c0 + 4 * ((int64_t)r * kPartThreads + threadIdx.x), n, kk, unused);
+        for (int u = 0; u < U; ++u) k[u] = q0 + u * stride < quads ? __ldcs(k4 + q0 + u * stride) : make_int4(-1, -1, -1, -1);
 #pragma unroll
-        for (int c = 0; c < 4; ++c)
-            if (in_range(kk[c], m)) atomicAdd(&s_cnt[bdiv((uint32_t)kk[c])], 1);
+        for (int u = 0; u < U; ++u) {
+            add(k[u].x);
+            add(k[u].y);
+            add(k[u].z);
+            add(k[u].w);
+        }
     }
+    if (blockIdx.x == 0 && 4 * quads + tid < n) add(keys[4 * quads + tid]);
     __syncthreads();
-    for (int b = threadIdx.x; b <= B; b += kPartThreads)
-        counts[(int64_t)b * nchunks + blockIdx.x] = b < B ? s_cnt[b] : 0;
+    for (int b = tid; b < B; b += kPartThreads)
+        if (s_cnt[b]) atomicAdd(totals + b, s_cnt[b]);
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    int32_t own[PER], sum = 0;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        const int b = tid * PER + j;
+        own[j] = b < B ? __ldcg(totals + b) : 0;
+        sum += own[j];
+    }
+    int32_t inc = sum;
+#pragma unroll
+    for (int o = 1; o < kWarp; o <<= 1) {
+        const int32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    if (lane == kWarp - 1) s_part[warp] = inc;
+    __syncthreads();
+    int32_t run = inc - sum;
+    for (int w = 0; w < warp; ++w) run += s_part[w];
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        const int b = tid * PER + j;
+        if (b <= B) start[b] = run;
+        if (b < B) cursor[b] = run;
+        run += own[j];
+    }
+    if (tid == kPartThreads - 1 && B == kPartMaxBuckets) start[B] = run;
 }
 
 // 3. Counting sort of one chunk by bucket in shared memory, then contiguous
-// runs out: obin = bin - bucket * W, oval = payload, at offs[b][chunk] + rank.
+// runs out: obin = bin - bucket * W, oval = payload, in the run that the chunk
+// reserves at its bucket's cursor.
 // Register-lean so that two blocks fit an SM: a thread keeps only each
 // element's (bucket, bin) word and its 16-bit rank, and reloads the values
 // (just read, so L1/L2 hits) when it places the elements.
 template <typename T, int MODE>
 __global__ void __launch_bounds__(kPartThreads, 2)
 k_part_scatter(const int32_t *__restrict__ keys, const T *__restrict__ vals, const int64_t n, const int64_t m,
-               const BucketDiv bdiv, const int B, const int64_t nchunks, const int32_t *__restrict__ offs,
-               uint16_t *__restrict__ obin, typename PartTraits<T, MODE>::V *__restrict__ oval) {
+               const BucketDiv bdiv, const int B, int32_t *__restrict__ cursor, uint16_t *__restrict__ obin,
+               typename PartTraits<T, MODE>::V *__restrict__ oval) {
     using Tr = PartTraits<T, MODE>;
     using V = typename Tr::V;
     constexpr int NW = kPartThreads / kWarp;
@@ -337,7 +387,7 @@ k_part_scatter(const int32_t *__restrict__ keys, const T *__restrict__ vals, con
         const int b = tid * PER + j;
         if (b < B) {
             s_loc[b] = run;
-            s_dst[b] = offs[(int64_t)b * nchunks + c] - run;
+            s_dst[b] = (own[j] ? atomicAdd(cursor + b, own[j]) : 0) - run;
             run += own[j];
         }
     }
@@ -373,22 +423,25 @@ k_part_scatter(const int32_t *__restrict__ keys, const T *__restrict__ vals, con
     }
 }
 
-// 3 (fp32). The same counting sort as a persistent, double-buffered pipeline:
-// block b owns chunks b, b + G, b + 2G, ... (G blocks, one per SM); each
-// whole chunk's keys and values arrive in shared memory by two bulk copies
-// issued one chunk ahead, so the DRAM reads of the next chunk overlap the
-// ranking, the bucket scan and the writes of this one.  The chunk is ranked
-// by bucket as above; a permutation of (bucket, element) words in bucket
-// order takes the place of the sorted payload copy, and the readout gathers
-// key and value from the staged chunk.  The ragged last chunk is loaded by plain loads.
+// 3 (fp32). The same counting sort with the chunk staged in shared memory:
+// persistent blocks, two per SM, each taking chunks b, b + G, ...; a whole
+// chunk's keys and values arrive by two bulk copies, and while one block waits
+// for its copy, ranks, scans or stores, the other one works (one block per SM
+// with the copies a chunk ahead spent its time in its own barriers: 6.6 us per
+// 8192-element chunk, issue slots half idle).  The elements are ranked with
+// shared-memory counters, a 16-bit permutation puts them in bucket order, and
+// the readout gathers key and value from the staged chunk; nothing but the
+// ranks stays in registers (the bucket of a key is recomputed), so 2048
+// threads fit.  The ragged last chunk is loaded by plain loads.
 constexpr int kScatThreads = 1024;
-static_assert(kPartChunk == (1 << 13), "the permutation word keeps the element in its low 13 bits");
+static_assert(kPartChunk <= (1 << 16), "the permutation holds 16-bit element numbers");
 constexpr int kScatItems = kPartChunk / kScatThreads;  // 8 elements per thread
+inline size_t scat_smem(int B) { return (size_t)kPartChunk * (4 + 4 + 2) + (size_t)B * 8; }
 
 template <int MODE>
-__global__ void __launch_bounds__(kScatThreads, 1)
+__global__ void __launch_bounds__(kScatThreads, 2)
 k_part_scatter_tma(const int32_t *__restrict__ keys, const float *__restrict__ vals, const int64_t n, const int64_t m,
-                   const BucketDiv bdiv, const int B, const int64_t nchunks, const int32_t *__restrict__ offs,
+                   const BucketDiv bdiv, const int B, const int64_t nchunks, int32_t *__restrict__ cursor,
                    uint16_t *__restrict__ obin, typename PartTraits<float, MODE>::V *__restrict__ oval,
                    unsigned *__restrict__ err, const long long spin_limit) {
     using Tr = PartTraits<float, MODE>;
@@ -396,52 +449,40 @@ k_part_scatter_tma(const int32_t *__restrict__ keys, const float *__restrict__ v
     constexpr int PER = kPartMaxBuckets / kScatThreads;  // buckets per thread in the local scan
     constexpr uint32_t kChunkBytes = kPartChunk * 4u;
     extern __shared__ __align__(16) unsigned char smem_raw[];  // bulk copies need 16-byte alignment
-    int32_t *const s_key0 = reinterpret_cast<int32_t *>(smem_raw);        // [2][kPartChunk] keys
-    float *const s_val0 = reinterpret_cast<float *>(s_key0 + 2 * kPartChunk);  // [2][kPartChunk] values
-    uint32_t *const s_perm = reinterpret_cast<uint32_t *>(s_val0 + 2 * kPartChunk);  // [kPartChunk] b << 13 | i
-    int32_t *const s_loc = reinterpret_cast<int32_t *>(s_perm + kPartChunk);        // [B]
-    int32_t *const s_dst = s_loc + B;                                                // [B]
-    __shared__ __align__(8) unsigned long long s_bar[2];
+    int32_t *const sk = reinterpret_cast<int32_t *>(smem_raw);             // [kPartChunk] keys
+    float *const sv = reinterpret_cast<float *>(sk + kPartChunk);          // [kPartChunk] values
+    uint16_t *const s_perm = reinterpret_cast<uint16_t *>(sv + kPartChunk);  // [kPartChunk] elements in bucket order
+    int32_t *const s_loc = reinterpret_cast<int32_t *>(s_perm + kPartChunk);  // [B] counts, then local starts
+    int32_t *const s_dst = s_loc + B;                                          // [B] global start - local start
+    __shared__ __align__(8) unsigned long long s_bar;
     __shared__ int32_t s_part[NW];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t G = gridDim.x;
     const auto whole = [&](int64_t c) { return (c + 1) * (int64_t)kPartChunk <= n; };
-    // thread 0: keys and values of chunk c into buffer `buf`
-    const auto issue = [&](int64_t c, int buf) {
+    const auto issue = [&](int64_t c) {  // thread 0
         fence_proxy_async_smem();
-        mbar_expect_tx(&s_bar[buf], 2u * kChunkBytes);
-        bulk_g2s(s_key0 + buf * kPartChunk, keys + c * kPartChunk, kChunkBytes, &s_bar[buf]);
-        bulk_g2s(s_val0 + buf * kPartChunk, vals + c * kPartChunk, kChunkBytes, &s_bar[buf]);
+        mbar_expect_tx(&s_bar, 2u * kChunkBytes);
+        bulk_g2s(sk, keys + c * kPartChunk, kChunkBytes, &s_bar);
+        bulk_g2s(sv, vals + c * kPartChunk, kChunkBytes, &s_bar);
     };
     if (tid == 0) {
-        mbar_init(&s_bar[0], 1);
-        mbar_init(&s_bar[1], 1);
+        mbar_init(&s_bar, 1);
         mbar_init_fence();
     }
     for (int b = tid; b < B; b += kScatThreads) s_loc[b] = 0;
     __syncthreads();
-    if (tid == 0 && (int64_t)blockIdx.x < nchunks && whole(blockIdx.x)) issue(blockIdx.x, 0);
-    uint32_t used0 = 0u, used1 = 0u;  // completed copy phases consumed, per buffer (same in every thread)
-    int j = 0;
-    for (int64_t c = blockIdx.x; c < nchunks; c += G, ++j) {
-        const int buf = j & 1;
-        const int64_t cn = c + G;
-        const bool next_staged = cn < nchunks && whole(cn);
-        if (tid == 0 && next_staged) issue(cn, buf ^ 1);  // that buffer's readers passed the last barrier
-        int32_t *const sk = s_key0 + buf * kPartChunk;
-        float *const sv = s_val0 + buf * kPartChunk;
+    if (tid == 0 && (int64_t)blockIdx.x < nchunks && whole(blockIdx.x)) issue(blockIdx.x);
+    uint32_t used = 0u;  // completed copies consumed (same in every thread)
+    for (int64_t c = blockIdx.x; c < nchunks; c += G) {
         const int64_t e0 = c * kPartChunk;
         const int len = (int)((n - e0) < kPartChunk ? (n - e0) : kPartChunk);
         if (whole(c)) {
-            const uint32_t mine = buf ? used1 : used0, other = buf ? used0 : used1;
-            const bool ok = mbar_wait_bounded(&s_bar[buf], mine & 1u, spin_limit);
-            if (buf) ++used1;
-            else ++used0;
-            if (!__syncthreads_and(ok)) {
-                // give up: report, let the copy in flight into the other buffer land, leave
+            const bool ok = mbar_wait_bounded(&s_bar, used & 1u, spin_limit);
+            ++used;
+            if (!__syncthreads_and(ok)) {  // report, give the copy a second bounded wait, leave
                 if (tid == 0) {
                     set_error(err, kErrTimeout);
-                    if (next_staged) mbar_wait_bounded(&s_bar[buf ^ 1], other & 1u, spin_limit);
+                    mbar_wait_bounded(&s_bar, (used - 1u) & 1u, spin_limit);
                 }
                 return;
             }
@@ -453,42 +494,29 @@ k_part_scatter_tma(const int32_t *__restrict__ keys, const float *__restrict__ v
             __syncthreads();
         }
 
-        // this chunk's run starts of the thread's buckets in the scan below: loaded
-        // now, so that their latency hides behind the ranking
-        int32_t gofs[PER];
-#pragma unroll
-        for (int q = 0; q < PER; ++q) {
-            const int b = tid * PER + q;
-            gofs[q] = b < B ? __ldg(offs + (int64_t)b * nchunks + c) : 0;
-        }
-
-        // rank every in-range element within its bucket
-        uint32_t bk[kScatItems];       // bucket << 16 | bin, or ~0u: absent or out of range
+        // rank every in-range element within its bucket (0xffff: out of range)
         uint32_t rk2[kScatItems / 2];  // two 16-bit ranks per word
 #pragma unroll
         for (int r = 0; r < kScatItems; ++r) {
             const int i = r * kScatThreads + tid;
-            uint32_t rank = 0;
-            bk[r] = 0xffffffffu;
+            uint32_t rank = 0xffffu;
             if (i < len) {
                 const int32_t k = sk[i];
-                if (in_range(k, m)) {
-                    const uint32_t b = bdiv((uint32_t)k);
-                    bk[r] = (b << 16) | ((uint32_t)k - b * bdiv.W);
-                    rank = (uint32_t)atomicAdd(&s_loc[b], 1);
-                }
+                if (in_range(k, m)) rank = (uint32_t)atomicAdd(&s_loc[bdiv((uint32_t)k)], 1);
             }
             if (r & 1) rk2[r >> 1] |= rank << 16;
             else rk2[r >> 1] = rank;
         }
         __syncthreads();
 
-        // exclusive scan of the B bucket counts (PER consecutive buckets per thread)
-        int32_t own[PER], sum = 0;
+        // reserve the chunk's runs at the buckets' cursors, and scan the bucket
+        // counts (PER consecutive buckets per thread)
+        int32_t own[PER], gofs[PER], sum = 0;
 #pragma unroll
         for (int q = 0; q < PER; ++q) {
             const int b = tid * PER + q;
             own[q] = b < B ? s_loc[b] : 0;
+            gofs[q] = own[q] ? atomicAdd(cursor + b, own[q]) : 0;
             sum += own[q];
         }
         int32_t inc = sum;
@@ -499,14 +527,15 @@ k_part_scatter_tma(const int32_t *__restrict__ keys, const float *__restrict__ v
         }
         if (lane == kWarp - 1) s_part[warp] = inc;
         __syncthreads();
-        int32_t before = 0, total = 0;
+        const int32_t wtot = s_part[lane];  // 32 warps, one per lane
+        int32_t winc = wtot;
 #pragma unroll
-        for (int w = 0; w < NW; ++w) {
-            const int32_t x = s_part[w];
-            if (w < warp) before += x;
-            total += x;
+        for (int o = 1; o < kWarp; o <<= 1) {
+            const int32_t y = __shfl_up_sync(0xffffffffu, winc, o);
+            if (lane >= o) winc += y;
         }
-        int32_t run = before + inc - sum;
+        const int32_t total = __shfl_sync(0xffffffffu, winc, 31);
+        int32_t run = __shfl_sync(0xffffffffu, winc - wtot, warp) + inc - sum;
 #pragma unroll
         for (int q = 0; q < PER; ++q) {
             const int b = tid * PER + q;
@@ -518,28 +547,27 @@ k_part_scatter_tma(const int32_t *__restrict__ keys, const float *__restrict__ v
         }
         __syncthreads();
 
-        // the permutation: position in bucket order -> (bucket, element of the chunk)
+        // the permutation: position in bucket order -> element of the chunk
 #pragma unroll
         for (int r = 0; r < kScatItems; ++r) {
-            if (bk[r] != 0xffffffffu) {
-                const uint32_t rank = (r & 1) ? (rk2[r >> 1] >> 16) : (rk2[r >> 1] & 0xffffu);
-                const uint32_t b = bk[r] >> 16;
-                s_perm[s_loc[b] + (int)rank] = (b << 13) | (uint32_t)(r * kScatThreads + tid);
-            }
+            const uint32_t rank = (r & 1) ? (rk2[r >> 1] >> 16) : (rk2[r >> 1] & 0xffffu);
+            const int i = r * kScatThreads + tid;
+            if (rank != 0xffffu) s_perm[s_loc[bdiv((uint32_t)sk[i])] + (int)rank] = (uint16_t)i;
         }
         __syncthreads();
 
         // contiguous runs out; the bucket counters are cleared for the next chunk
+        for (int b = tid; b < B; b += kScatThreads) s_loc[b] = 0;
         for (int pos = tid; pos < total; pos += kScatThreads) {
-            const uint32_t x = s_perm[pos];
-            const int i = (int)(x & (kPartChunk - 1));
-            const uint32_t b = x >> 13;
+            const int i = s_perm[pos];
+            const uint32_t k = (uint32_t)sk[i];
+            const uint32_t b = bdiv(k);
             const int32_t g = s_dst[b] + pos;  // < n < 2^31
-            obin[g] = (uint16_t)((uint32_t)sk[i] - b * bdiv.W);
+            obin[g] = (uint16_t)(k - b * bdiv.W);
             oval[g] = Tr::enc(sv[i], e0 + i);
         }
-        for (int b = tid; b < B; b += kScatThreads) s_loc[b] = 0;
         __syncthreads();
+        if (tid == 0 && c + G < nchunks && whole(c + G)) issue(c + G);
     }
 }
 
@@ -548,7 +576,7 @@ k_part_scatter_tma(const int32_t *__restrict__ keys, const float *__restrict__ v
 template <typename T, int MODE>
 __global__ void __launch_bounds__(kPartTableThreads)
 k_part_table(const uint16_t *__restrict__ obin, const typename PartTraits<T, MODE>::V *__restrict__ oval,
-             const int32_t *__restrict__ offs, const int64_t nchunks, const int64_t m, const uint32_t W,
+             const int32_t *__restrict__ bucket, const int64_t m, const uint32_t W,
              const PartOut<T> out, unsigned *__restrict__ err) {
     using Tr = PartTraits<T, MODE>;
     using V = typename Tr::V;
@@ -557,8 +585,8 @@ k_part_table(const uint16_t *__restrict__ obin, const typename PartTraits<T, MOD
     const int w = (int)((m - j0) < (int64_t)W ? (m - j0) : (int64_t)W);
     for (int t = threadIdx.x; t < w; t += kPartTableThreads) Tr::init(smem_raw, (int)W, t);
     __syncthreads();
-    const int64_t start = offs[(int64_t)blockIdx.x * nchunks];
-    const int64_t end = offs[(int64_t)(blockIdx.x + 1) * nchunks];
+    const int64_t start = bucket[blockIdx.x];
+    const int64_t end = bucket[blockIdx.x + 1];
     constexpr int U = 8;
     for (int64_t g0 = start; g0 < end; g0 += (int64_t)U * kPartTableThreads) {
         int32_t u[U];
@@ -626,19 +654,16 @@ bool part_applicable(int mode, size_t s, int64_t m) {
 }
 
 struct PartLayout {
-    size_t counts, offs, scanreg, obin, oval, bytes;
+    size_t totals, start, cursor, obin, oval, bytes;
 };
 static PartLayout part_layout(const PartPlan &P, size_t payload, int64_t n) {
     PartLayout L;
-    const int64_t cells = (int64_t)(P.B + 1) * P.nchunks;
+    const size_t row = align_up((size_t)(P.B + 1) * 4, 256);
     size_t o = 0;
-    L.counts = o;
-    o = align_up(o + (size_t)cells * 4, 256);
-    L.offs = o;
-    o = align_up(o + (size_t)cells * 4, 256);
-    L.scanreg = o;
-    o = align_up(o + excl_scan_i32_region(cells), 256);
-    L.obin = o;
+    L.totals = o;
+    L.start = o += row;
+    L.cursor = o += row;
+    L.obin = o += row;
     o = align_up(o + (size_t)n * 2, 256);
     L.oval = o;
     o = align_up(o + (size_t)n * payload, 256);
@@ -665,36 +690,37 @@ static adc_status part_run(int64_t n, int64_t m, const int32_t *keys, const T *v
     if (!P.ok) return ADC_ERR_UNSUPPORTED;
     const PartLayout L = part_layout(P, sizeof(V), n);
     char *w = static_cast<char *>(ws) + ws_off;
-    int32_t *counts = reinterpret_cast<int32_t *>(w + L.counts);
-    int32_t *offs = reinterpret_cast<int32_t *>(w + L.offs);
+    int32_t *totals = reinterpret_cast<int32_t *>(w + L.totals);
+    int32_t *start = reinterpret_cast<int32_t *>(w + L.start);
+    int32_t *cursor = reinterpret_cast<int32_t *>(w + L.cursor);
     uint16_t *obin = reinterpret_cast<uint16_t *>(w + L.obin);
     V *oval = reinterpret_cast<V *>(w + L.oval);
     unsigned *err = reinterpret_cast<unsigned *>(ws);
     const int64_t nc = P.nchunks;
 
     const BucketDiv bdiv{P.W, P.inv};
-    k_part_count<<<(unsigned)nc, kPartThreads, (size_t)P.B * 4, s>>>(keys, n, m, bdiv, P.B, nc, counts);
+    if (cudaMemsetAsync(totals, 0, (size_t)P.B * 4, s) != cudaSuccess) return ADC_ERR_CUDA;
+    const int64_t gc = (n / 4 + kPartThreads - 1) / kPartThreads, cap = (int64_t)num_sms() * 4;
+    k_part_count<<<(unsigned)(gc < 1 ? 1 : gc < cap ? gc : cap), kPartThreads, (size_t)P.B * 4, s>>>(
+        keys, n, m, bdiv, P.B, totals, start, cursor, counter_slot(ws, kPartSlot));
     adc_status st = check_launch();
     if (st != ADC_OK) return st;
-    st = excl_scan_i32(counts, offs, (int64_t)(P.B + 1) * nc, ws, kPartSlot, w + L.scanreg, s);
-    if (st != ADC_OK) return st;
     if constexpr (sizeof(T) == 4) {
-        // staged pipeline: 2 x (keys + values) + the permutation + the bucket arrays
-        const size_t sm_tma = (size_t)kPartChunk * (4 * 4 + 4) + (size_t)P.B * 8;
+        const size_t sm_tma = scat_smem(P.B);
         if (!smem_attr(k_part_scatter_tma<MODE>, sm_tma)) return ADC_ERR_CUDA;
-        const int64_t grid = nc < num_sms() ? nc : num_sms();
-        k_part_scatter_tma<MODE><<<(unsigned)grid, kScatThreads, sm_tma, s>>>(keys, vals, n, m, bdiv, P.B, nc, offs,
-                                                                             obin, oval, err, spin_limit());
+        const int64_t two = (int64_t)num_sms() * 2;
+        k_part_scatter_tma<MODE><<<(unsigned)(nc < two ? nc : two), kScatThreads, sm_tma, s>>>(
+            keys, vals, n, m, bdiv, P.B, nc, cursor, obin, oval, err, spin_limit());
     } else {
         const size_t sm_scatter = (size_t)kPartChunk * (sizeof(V) + 4) + (size_t)P.B * 8;
         if (!smem_attr(k_part_scatter<T, MODE>, sm_scatter)) return ADC_ERR_CUDA;
-        k_part_scatter<T, MODE><<<(unsigned)nc, kPartThreads, sm_scatter, s>>>(keys, vals, n, m, bdiv, P.B, nc, offs,
+        k_part_scatter<T, MODE><<<(unsigned)nc, kPartThreads, sm_scatter, s>>>(keys, vals, n, m, bdiv, P.B, cursor,
                                                                               obin, oval);
     }
     if ((st = check_launch()) != ADC_OK) return st;
     const size_t sm_table = (size_t)P.W * Tr::kEntry;
     if (!smem_attr(k_part_table<T, MODE>, sm_table)) return ADC_ERR_CUDA;
-    k_part_table<T, MODE><<<(unsigned)P.B, kPartTableThreads, sm_table, s>>>(obin, oval, offs, nc, m, P.W, out, err);
+    k_part_table<T, MODE><<<(unsigned)P.B, kPartTableThreads, sm_table, s>>>(obin, oval, start, m, P.W, out, err);
     return check_launch();
 }
 
