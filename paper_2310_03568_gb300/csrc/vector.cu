@@ -879,16 +879,17 @@ __device__ __forceinline__ typename Op::S warp_parts_scan(const Op &op, typename
 
 template <class Op, int RP>
 __global__ void __launch_bounds__(kVScanThreads)
-k_vscan_wfold(const Op op, const int64_t n, const int64_t d, const int64_t U, typename Op::S *__restrict__ agg) {
+k_vscan_wfold(const Op op, const int64_t n, const int64_t d, const int64_t U, typename Op::S *__restrict__ before,
+              typename Op::S *__restrict__ agg) {
     using S = typename Op::S;
+    __shared__ S s_unit[kVScanWarps][kWarp];
     const int lane = threadIdx.x & 31;
     const int64_t u = (int64_t)blockIdx.x * kVScanWarps + (threadIdx.x >> 5);
-    if (u >= U) return;  // whole warps
     const int P = kWarp / (int)d;
-    const bool active = lane < P * (int)d;
+    const bool active = lane < P * (int)d && u < U;
     const int64_t c = lane % d, p = lane / d;
-    int64_t l0, l1;
-    vscan_range(n, u, U, &l0, &l1);
+    int64_t l0 = 0, l1 = 0;
+    if (u < U) vscan_range(n, u, U, &l0, &l1);
     S a = op.identity();
     if (active) {
         // part p folds a contiguous piece of the unit, RP loads in flight
@@ -912,23 +913,39 @@ k_vscan_wfold(const Op op, const int64_t n, const int64_t d, const int64_t U, ty
         }
     }
     a = warp_parts_scan(op, a, (int)d, P);
-    if (active && p == P - 1) agg[u * d + c] = a;
+    if (lane < P * (int)d && p == P - 1) s_unit[threadIdx.x >> 5][c] = a;
+    __syncthreads();
+    if (threadIdx.x < d) {  // one thread per column: the block's units in order
+        const int64_t t = threadIdx.x;
+        S run = op.identity();
+#pragma unroll
+        for (int w = 0; w < kVScanWarps; ++w) {
+            const int64_t uw = (int64_t)blockIdx.x * kVScanWarps + w;
+            if (uw < U) before[uw * d + t] = run;
+            run = op.combine(run, s_unit[w][t]);
+        }
+        agg[t * gridDim.x + blockIdx.x] = run;
+    }
 }
 
-// One block per column: the exclusive prefixes of the U unit states, in order.
+// One block per column: agg[c][g] (the G blocks' states of column c, next to
+// each other) become their exclusive prefixes, in place.  Per block and not per
+// unit, and column by column, because this kernel is a chain of latencies: at
+// d = 16 and about 9700 units, reading every unit's state at a stride of d
+// states took 28 us.
 constexpr int kVPrefixThreads = 1024;
 template <class Op>
 __global__ void __launch_bounds__(kVPrefixThreads)
-k_vscan_wprefix(const Op op, const typename Op::S *__restrict__ agg, const int64_t U, const int64_t d,
-                typename Op::S *__restrict__ pre) {
+k_vscan_wprefix(const Op op, typename Op::S *__restrict__ agg, const int64_t G) {
     using S = typename Op::S;
     __shared__ S s_w[kVPrefixThreads / kWarp];
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const int64_t c = blockIdx.x;
-    const int64_t per = (U + kVPrefixThreads - 1) / kVPrefixThreads;
-    const int64_t g0 = t * per, g1 = g0 + per < U ? g0 + per : U;
+    S *col = agg + c * G;
+    const int64_t per = (G + kVPrefixThreads - 1) / kVPrefixThreads;
+    const int64_t g0 = t * per < G ? t * per : G, g1 = g0 + per < G ? g0 + per : G;
     S v = op.identity();
-    for (int64_t g = g0; g < g1; ++g) v = op.combine(v, agg[g * d + c]);
+    for (int64_t g = g0; g < g1; ++g) v = op.combine(v, col[g]);
     const S inc = warp_inclusive_scan(op, v);
     if (lane == kWarp - 1) s_w[w] = inc;
     __syncthreads();
@@ -937,14 +954,16 @@ k_vscan_wprefix(const Op op, const typename Op::S *__restrict__ agg, const int64
     S ex = shfl_up(inc, 1);
     if (lane > 0) run = op.combine(run, ex);
     for (int64_t g = g0; g < g1; ++g) {
-        pre[g * d + c] = run;
-        run = op.combine(run, agg[g * d + c]);
+        const S x = col[g];
+        col[g] = run;
+        run = op.combine(run, x);
     }
 }
 
 template <class Op, int RP>
 __global__ void __launch_bounds__(kVScanThreads)
-k_vscan_wapply(const Op op, const int64_t n, const int64_t d, const int64_t U, const typename Op::S *__restrict__ pre) {
+k_vscan_wapply(const Op op, const int64_t n, const int64_t d, const int64_t U,
+               const typename Op::S *__restrict__ before, const typename Op::S *__restrict__ pre) {
     using S = typename Op::S;
     const int lane = threadIdx.x & 31;
     const int64_t u = (int64_t)blockIdx.x * kVScanWarps + (threadIdx.x >> 5);
@@ -955,7 +974,7 @@ k_vscan_wapply(const Op op, const int64_t n, const int64_t d, const int64_t U, c
     const int last = (P - 1) * (int)d + (int)c;  // the lane with column c's tile total
     int64_t l0, l1;
     vscan_range(n, u, U, &l0, &l1);
-    S carry = active ? pre[u * d + c] : op.identity();
+    S carry = active ? op.combine(pre[c * gridDim.x + blockIdx.x], before[u * d + c]) : op.identity();
     for (int64_t lt = l0; lt < l1; lt += (int64_t)P * RP) {
         const int64_t lp = lt + p * RP;
         S st[RP];
@@ -1006,9 +1025,9 @@ template <class Op, int RP> static adc_status vscan_run(const Op &op, int64_t n,
     if (d <= kWarp) {
         const int64_t U = vscan_units<Op, RP, true>(n);
         const unsigned blocks = (unsigned)((U + kVScanWarps - 1) / kVScanWarps);
-        k_vscan_wfold<Op, RP><<<blocks, kVScanThreads, 0, s>>>(op, n, d, U, agg);
-        k_vscan_wprefix<Op><<<(unsigned)d, kVPrefixThreads, 0, s>>>(op, agg, U, d, pre);
-        k_vscan_wapply<Op, RP><<<blocks, kVScanThreads, 0, s>>>(op, n, d, U, pre);
+        k_vscan_wfold<Op, RP><<<blocks, kVScanThreads, 0, s>>>(op, n, d, U, agg, pre);
+        k_vscan_wprefix<Op><<<(unsigned)d, kVPrefixThreads, 0, s>>>(op, pre, blocks);
+        k_vscan_wapply<Op, RP><<<blocks, kVScanThreads, 0, s>>>(op, n, d, U, agg, pre);
     } else {
         const int G = (int)vscan_units<Op, RP, false>(n);
         k_vscan_fold<Op, RP><<<G, kVScanThreads, 0, s>>>(op, n, d, agg);
