@@ -87,16 +87,21 @@ template <typename T, int Q> struct GMMQ {
 };
 
 // ------------------------------------------------------- simple reduction --
-// Workspace: [header][ticket u32 @ +8 in header][partials G states]
+// Workspace: [header][ticket u32 in header][partials G states]
 // The operators here (+, the lifted * and min/max, sumOfProd) are
 // commutative, so a thread may take any of the tile's elements: it takes
 // 16-byte words t, t + kRedThreads, ..., so that a warp's load covers 512
 // contiguous bytes.  The lifted operators get each element's own index.
-template <class Op, typename T, int ITEMS>
-__global__ void __launch_bounds__(kRedThreads)
-k_reduce_simple(const Op op, const T *__restrict__ x, const int64_t n, const int64_t tiles_per_block,
-                typename Op::State *__restrict__ part, unsigned *__restrict__ ticket,
-                typename Op::State *__restrict__ result) {
+// Bound by bytes in flight: kRedBlocksPerSM blocks of 256 threads with 64
+// bytes each per thread; whole tiles take no bounds checks.  The last block to
+// finish combines the partials in block order and writes y and the residuals
+// (`fin`), so there is no launch after this one.
+constexpr int kRedBlocksPerSM = 6;
+
+template <class Op, class Fin, typename T, int ITEMS>
+__global__ void __launch_bounds__(kRedThreads, kRedBlocksPerSM)
+k_reduce_simple(const Op op, const Fin fin, const T *__restrict__ x, const int64_t n, const int64_t tiles_per_block,
+                typename Op::State *__restrict__ part, unsigned *__restrict__ ticket) {
     using S = typename Op::State;
     constexpr int TILE = kRedThreads * ITEMS;
     constexpr int WE = 16 / sizeof(T) < ITEMS ? 16 / sizeof(T) : ITEMS;  // elements per word
@@ -108,15 +113,26 @@ k_reduce_simple(const Op op, const T *__restrict__ x, const int64_t n, const int
     for (int64_t t = t0; t < t0 + tiles_per_block; ++t) {
         if (t * TILE >= n) break;
         T v[NWD][WE];
-#pragma unroll
-        for (int j = 0; j < NWD; ++j)
-            load_chunk(x, t * TILE + ((int64_t)j * kRedThreads + threadIdx.x) * WE, n, v[j], T{});
+        const bool whole = (t + 1) * TILE <= n;
 #pragma unroll
         for (int j = 0; j < NWD; ++j) {
             const int64_t c0 = t * TILE + ((int64_t)j * kRedThreads + threadIdx.x) * WE;
+            load_chunk(x, c0, whole ? c0 + WE : n, v[j], T{});
+        }
+        const int64_t b0 = t * TILE + (int64_t)threadIdx.x * WE;
+        if (whole) {
 #pragma unroll
-            for (int k = 0; k < WE; ++k)
-                if (c0 + k < n) acc = op.combine(acc, op.lift(v[j][k], c0 + k));
+            for (int j = 0; j < NWD; ++j)
+#pragma unroll
+                for (int k = 0; k < WE; ++k) acc = op.combine(acc, op.lift(v[j][k], b0 + j * kRedThreads * WE + k));
+        } else {
+#pragma unroll
+            for (int j = 0; j < NWD; ++j)
+#pragma unroll
+                for (int k = 0; k < WE; ++k) {
+                    const int64_t i = b0 + j * kRedThreads * WE + k;
+                    if (i < n) acc = op.combine(acc, op.lift(v[j][k], i));
+                }
         }
     }
     S total;
@@ -137,21 +153,32 @@ k_reduce_simple(const Op op, const T *__restrict__ x, const int64_t n, const int
         if (b < (int)gridDim.x) a = op.combine(a, load_cg(&part[b]));
     }
     block_exclusive_fwd<Op, kRedThreads>(op, a, tmp, &total);
-    if (threadIdx.x == 0) *result = total;
+    if (threadIdx.x == 0) fin(total);
 }
 
-// Finalisers: turn the lifted result into y and the saved residuals.
-template <typename T> __global__ void k_fin_add(const T *r, T *y) { *y = *r; }
-template <typename T> __global__ void k_fin_sel(const MinMaxS<T> *r, T *y, int32_t *k) {
-    *y = r->v;
-    *k = r->i;
-}
-template <typename T> __global__ void k_fin_sop(const Pair<T> *r, Pair<T> *y) { *y = *r; }
-template <typename T> __global__ void k_fin_mul(const MulS<T> *r, T *y, int32_t *n0, T *p) {
-    *y = r->z > 0 ? T(0) : r->p;
-    *n0 = r->z;
-    *p = r->p;
-}
+// What the last block does with the lifted result: y and the saved residuals.
+template <typename T> struct FinAdd {
+    T *y;
+    __device__ void operator()(const T &r) const { *y = r; }
+};
+template <typename T> struct FinSel {
+    T *y;
+    int32_t *k;
+    __device__ void operator()(const MinMaxS<T> &r) const {
+        *y = r.v;
+        *k = r.i;
+    }
+};
+template <typename T> struct FinMul {
+    T *y;
+    int32_t *n0;
+    T *p;
+    __device__ void operator()(const MulS<T> &r) const {
+        *y = r.z > 0 ? T(0) : r.p;
+        *n0 = r.z;
+        *p = r.p;
+    }
+};
 
 // ------------------------------------------------------ general reduction --
 // Pass 1: the aggregate of every tile, in order.
@@ -414,7 +441,7 @@ static bool is_general(adc_op op) {
 }
 
 static int64_t simple_grid(int64_t tiles) {
-    int64_t g = (int64_t)num_sms() * 4;
+    int64_t g = (int64_t)num_sms() * kRedBlocksPerSM;
     if (tiles < g) g = tiles;
     return g < 1 ? 1 : g;
 }
@@ -504,18 +531,15 @@ size_t reduce_saved_bytes(adc_op op, adc_dtype dt, int64_t n) {
     return dt == ADC_F64 ? red_saved_t<double>(op, n) : red_saved_t<float>(op, n);
 }
 
-template <class Op, typename T, int ITEMS>
-static adc_status launch_simple(const Op &op, const T *x, int64_t n, void *ws, cudaStream_t s,
-                                typename Op::State **result) {
+template <class Op, typename T, int ITEMS, class Fin>
+static adc_status launch_simple(const Op &op, const Fin &fin, const T *x, int64_t n, void *ws, cudaStream_t s) {
     constexpr int TILE = kRedThreads * ITEMS;
     const int64_t tiles = (n + TILE - 1) / TILE;
     const int64_t G = simple_grid(tiles);
     const int64_t tpb = tiles > 0 ? (tiles + G - 1) / G : 0;
-    char *w = static_cast<char *>(ws);
-    auto *part = reinterpret_cast<typename Op::State *>(w + kWsHeader);
-    *result = part + G;
-    k_reduce_simple<Op, T, ITEMS><<<(unsigned)G, kRedThreads, 0, s>>>(op, x, n, tpb, part, counter_slot(ws, 1),
-                                                                       *result);
+    auto *part = reinterpret_cast<typename Op::State *>(static_cast<char *>(ws) + kWsHeader);
+    k_reduce_simple<Op, Fin, T, ITEMS><<<(unsigned)G, kRedThreads, 0, s>>>(op, fin, x, n, tpb, part,
+                                                                            counter_slot(ws, 1));
     return check_launch();
 }
 
@@ -524,45 +548,17 @@ static adc_status red_fwd_t(adc_op op, int64_t n, const void *xv, void *yv, void
     constexpr int I = RedItems<T>::scalar;
     const T *x = static_cast<const T *>(xv);
     T *y = static_cast<T *>(yv);
-    adc_status st;
+    int32_t *k = static_cast<int32_t *>(saved);
     switch (op) {
-    case ADC_OP_ADD: {
-        RAdd<T> o;
-        T *r;
-        if ((st = launch_simple<RAdd<T>, T, I>(o, x, n, ws, s, &r)) != ADC_OK) return st;
-        k_fin_add<T><<<1, 1, 0, s>>>(r, y);
-        return check_launch();
-    }
-    case ADC_OP_MIN:
-    case ADC_OP_MAX: {
-        MinMaxS<T> *r;
-        if (op == ADC_OP_MIN) {
-            RSel<T, false> o{(int32_t)n};
-            if ((st = launch_simple<RSel<T, false>, T, I>(o, x, n, ws, s, &r)) != ADC_OK) return st;
-        } else {
-            RSel<T, true> o{(int32_t)n};
-            if ((st = launch_simple<RSel<T, true>, T, I>(o, x, n, ws, s, &r)) != ADC_OK) return st;
-        }
-        k_fin_sel<T><<<1, 1, 0, s>>>(r, y, static_cast<int32_t *>(saved));
-        return check_launch();
-    }
-    case ADC_OP_MUL: {
-        RMul<T> o;
-        MulS<T> *r;
-        if ((st = launch_simple<RMul<T>, T, I>(o, x, n, ws, s, &r)) != ADC_OK) return st;
-        k_fin_mul<T><<<1, 1, 0, s>>>(r, y, static_cast<int32_t *>(saved),
-                                     reinterpret_cast<T *>(static_cast<char *>(saved) + 8));
-        return check_launch();
-    }
-    case ADC_OP_SOP: {
-        RSop<T> o;
-        Pair<T> *r;
-        if ((st = launch_simple<RSop<T>, Pair<T>, RedItems<T>::pair>(o, static_cast<const Pair<T> *>(xv), n, ws, s,
-                                                                     &r)) != ADC_OK)
-            return st;
-        k_fin_sop<T><<<1, 1, 0, s>>>(r, static_cast<Pair<T> *>(yv));
-        return check_launch();
-    }
+    case ADC_OP_ADD: return launch_simple<RAdd<T>, T, I>(RAdd<T>{}, FinAdd<T>{y}, x, n, ws, s);
+    case ADC_OP_MIN: return launch_simple<RSel<T, false>, T, I>(RSel<T, false>{(int32_t)n}, FinSel<T>{y, k}, x, n, ws, s);
+    case ADC_OP_MAX: return launch_simple<RSel<T, true>, T, I>(RSel<T, true>{(int32_t)n}, FinSel<T>{y, k}, x, n, ws, s);
+    case ADC_OP_MUL:
+        return launch_simple<RMul<T>, T, I>(
+            RMul<T>{}, FinMul<T>{y, k, reinterpret_cast<T *>(static_cast<char *>(saved) + 8)}, x, n, ws, s);
+    case ADC_OP_SOP:
+        return launch_simple<RSop<T>, Pair<T>, RedItems<T>::pair>(RSop<T>{}, FinAdd<Pair<T>>{static_cast<Pair<T> *>(yv)},
+                                                                 static_cast<const Pair<T> *>(xv), n, ws, s);
     case ADC_OP_LIN:
         return general_fwd<GLin<T>, T, RedItems<T>::pair>(n, xv, yv, saved, ws, s);
     case ADC_OP_MM2:
