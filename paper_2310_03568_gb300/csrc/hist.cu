@@ -1229,6 +1229,57 @@ __global__ void k_hist_mul_vjp(const int32_t *__restrict__ keys, const T *__rest
     }
 }
 
+// The same with the coefficient table of a bin count beyond L1 but within a
+// block in shared memory (one 1024-thread block per SM; the rare zeros read
+// the second table from L2): a gather that missed L1 cost an L2 round trip per
+// element.
+template <typename T>
+__global__ void __launch_bounds__(1024, 1)
+k_hist_mul_vjp_smem(const int32_t *__restrict__ keys, const T *__restrict__ vals, const T *__restrict__ anz,
+                    const T *__restrict__ az, T *__restrict__ vb, const int64_t n, const int64_t m,
+                    const int accumulate) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T *tab = reinterpret_cast<T *>(smem_raw);
+    for (int64_t j = threadIdx.x; j < m; j += blockDim.x) tab[j] = anz[j];
+    __syncthreads();
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    auto grad = [&](int32_t k, T v) -> T {
+        if (!in_range(k, m)) return T(0);
+        return v != T(0) ? div_or_zero(tab[k], v) : __ldg(az + k);
+    };
+    constexpr int U = sizeof(T) == 4 ? 4 : 2;  // 4-element groups per thread and step: all their loads issued first
+    const int64_t nv = n / 4;
+    for (int64_t v0 = g; v0 < nv; v0 += U * stride) {
+        int4 k[U];
+        T a[U][4];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t v = v0 + u * stride;
+            k[u] = v < nv ? __ldcs(reinterpret_cast<const int4 *>(keys) + v) : make_int4(-1, -1, -1, -1);
+            load_chunk_cs(vals, v * 4, v < nv ? n : 0, a[u], T(1));
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t v = v0 + u * stride;
+            if (v >= nv) break;
+            T o[4];
+            if (accumulate) load_chunk(vb, v * 4, n, o, T(0));
+            const int kk[4] = {k[u].x, k[u].y, k[u].z, k[u].w};
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const T gv = grad(kk[c], a[u][c]);
+                o[c] = accumulate ? o[c] + gv : gv;
+            }
+            store_chunk(vb, v * 4, n, o);
+        }
+    }
+    for (int64_t i = nv * 4 + g; i < n; i += stride) {
+        const T gv = grad(keys[i], vals[i]);
+        vb[i] = accumulate ? vb[i] + gv : gv;
+    }
+}
+
 template <typename T>
 __global__ void k_h0bar_mul(const int32_t *__restrict__ n0, const T *__restrict__ p, const T *__restrict__ hb,
                             T *__restrict__ h0b, const int64_t m, const int accumulate) {
@@ -1765,7 +1816,15 @@ static adc_status hist_vjp_t(adc_op op, int64_t n, int64_t m, const int32_t *key
         T *az = reinterpret_cast<T *>(static_cast<char *>(ws) + kWsHeader + align_up((size_t)m * sizeof(T), 256));
         if (n > 0) {
             k_mul_vjp_prep<T><<<gm, 256, 0, s>>>(n0, p, h0, hb, anz, az, m);
-            k_hist_mul_vjp<T><<<gn8, 256, 0, s>>>(keys, vals, anz, az, vb, n, m, acc);
+            // a table that misses L1 but fits a block, and enough elements to pay for
+            // loading it into every SM
+            const size_t tab = (size_t)m * sizeof(T);
+            if (tab > 64 * 1024 && tab <= kBlockBudget && n >= 64 * m) {
+                if (!set_smem(k_hist_mul_vjp_smem<T>, tab)) return ADC_ERR_CUDA;
+                k_hist_mul_vjp_smem<T><<<num_sms(), 1024, tab, s>>>(keys, vals, anz, az, vb, n, m, acc);
+            } else {
+                k_hist_mul_vjp<T><<<gn8, 256, 0, s>>>(keys, vals, anz, az, vb, n, m, acc);
+            }
         }
         if (h0b) k_h0bar_mul<T><<<gm, 256, 0, s>>>(n0, p, hb, h0b, m, acc);
         return check_launch();
