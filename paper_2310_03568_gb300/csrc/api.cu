@@ -66,9 +66,12 @@ bool one_ok(const void *p, adc_dtype dt) { return p != nullptr && aligned(p, dt 
 
 cudaStream_t as_stream(void *s) { return static_cast<cudaStream_t>(s); }
 
-adc_status prologue(void *ws, size_t ws_bytes, size_t need, cudaStream_t s) {
+// `zero`: zero the workspace's header here; the calls that pass false do it with
+// their first memset or kernel (a launch less, which is what a small call costs).
+adc_status prologue(void *ws, size_t ws_bytes, size_t need, cudaStream_t s, bool zero = true) {
     if (ws == nullptr || !aligned(ws, 256)) return ADC_ERR_INVALID_ARG;
     if (ws_bytes < need) return ADC_ERR_WORKSPACE;
+    if (!zero) return ADC_OK;
     if (cudaMemsetAsync(ws, 0, kWsHeader, s) != cudaSuccess) return ADC_ERR_CUDA;
     return ADC_OK;
 }
@@ -164,7 +167,7 @@ adc_status adc_reduce_vjp(adc_op op, adc_dtype dt, int64_t n, const void *x, con
     if (op == ADC_OP_SOP && !one_ok(y, dt)) return ADC_ERR_INVALID_ARG;
     if (op != ADC_OP_ADD && op != ADC_OP_SOP && (saved == nullptr || !aligned(saved, 16))) return ADC_ERR_INVALID_ARG;
     cudaStream_t s = as_stream(stream);
-    adc_status st = prologue(ws, ws_bytes, reduce_ws_bytes(op, dt, n), s);
+    adc_status st = prologue(ws, ws_bytes, reduce_ws_bytes(op, dt, n), s, false);
     if (st != ADC_OK) return st;
     return reduce_vjp(op, dt, n, x, y, saved, ybar, xbar, accumulate ? 1 : 0, ws, s);
 }
@@ -175,7 +178,7 @@ adc_status adc_scan_fwd(adc_op op, adc_dtype dt, int64_t n, const void *x, void 
     if (!scan_op(op)) return ADC_ERR_UNSUPPORTED;
     if (!arr_ok(x, n) || !arr_ok(y, n)) return ADC_ERR_INVALID_ARG;
     cudaStream_t s = as_stream(stream);
-    adc_status st = prologue(ws, ws_bytes, scan_ws_bytes(op, dt, n), s);
+    adc_status st = prologue(ws, ws_bytes, scan_ws_bytes(op, dt, n), s, false);
     if (st != ADC_OK) return st;
     return scan_fwd(op, dt, n, x, y, ws, s);
 }
@@ -187,7 +190,7 @@ adc_status adc_scan_vjp(adc_op op, adc_dtype dt, int64_t n, const void *x, const
     if (!arr_ok(ybar, n) || !arr_ok(xbar, n)) return ADC_ERR_INVALID_ARG;
     if (op != ADC_OP_ADD && (!arr_ok(x, n) || !arr_ok(y, n))) return ADC_ERR_INVALID_ARG;
     cudaStream_t s = as_stream(stream);
-    adc_status st = prologue(ws, ws_bytes, scan_ws_bytes(op, dt, n), s);
+    adc_status st = prologue(ws, ws_bytes, scan_ws_bytes(op, dt, n), s, false);
     if (st != ADC_OK) return st;
     return scan_vjp(op, dt, n, x, y, ybar, xbar, accumulate ? 1 : 0, ws, s);
 }
@@ -203,7 +206,7 @@ adc_status adc_hist_fwd(adc_op op, adc_dtype dt, int64_t n, int64_t m, const int
     if (op == ADC_OP_LIN && saved == nullptr) return ADC_ERR_INVALID_ARG;
     if (saved != nullptr && !aligned(saved, 16)) return ADC_ERR_INVALID_ARG;
     cudaStream_t s = as_stream(stream);
-    adc_status st = prologue(ws, ws_bytes, hist_ws_bytes(op, dt, n, m), s);
+    adc_status st = prologue(ws, ws_bytes, hist_ws_bytes(op, dt, n, m), s, op != ADC_OP_ADD);
     if (st != ADC_OK) return st;
     return hist_fwd(op, dt, n, m, keys, vals, hist0, hist, saved, ws, s);
 }
@@ -222,7 +225,7 @@ adc_status adc_hist_vjp(adc_op op, adc_dtype dt, int64_t n, int64_t m, const int
         return ADC_ERR_INVALID_ARG;
     if (op != ADC_OP_ADD && op != ADC_OP_SOP && (saved == nullptr || !aligned(saved, 16))) return ADC_ERR_INVALID_ARG;
     cudaStream_t s = as_stream(stream);
-    adc_status st = prologue(ws, ws_bytes, hist_ws_bytes(op, dt, n, m), s);
+    adc_status st = prologue(ws, ws_bytes, hist_ws_bytes(op, dt, n, m), s, op != ADC_OP_ADD);
     if (st != ADC_OK) return st;
     return hist_vjp(op, dt, n, m, keys, vals, hist0, hist, saved, histbar, valsbar, hist0bar, accumulate ? 1 : 0, ws,
                     s);

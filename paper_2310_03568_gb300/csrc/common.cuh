@@ -7,6 +7,7 @@
 #include <stdint.h>
 
 #include "../../include/adcomb.h"
+#include "internal.h"
 
 namespace adc {
 
@@ -36,6 +37,11 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *p) {
 
 __device__ __forceinline__ void st_release_u32(unsigned *p, unsigned v) {
     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+// Zeroes the workspace's header from a kernel that uses none of it.
+__device__ __forceinline__ void zero_header(unsigned *header) {
+    if (blockIdx.x == 0 && threadIdx.x < kWsHeader / 4) header[threadIdx.x] = 0u;
 }
 
 __device__ __forceinline__ void set_error(unsigned *err, unsigned bit) { atomicOr(err, bit); }

@@ -141,7 +141,9 @@ __device__ __forceinline__ void for_each_batch(const int32_t *__restrict__ keys,
 
 // ===================================================================== ADD ==
 template <typename T>
-__global__ void k_hist_init(T *__restrict__ h, const T *__restrict__ h0, const int64_t m, const T e) {
+__global__ void k_hist_init(T *__restrict__ h, const T *__restrict__ h0, const int64_t m, const T e,
+                            unsigned *__restrict__ header) {
+    if (header) zero_header(header);
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x)
         h[j] = h0 ? h0[j] : e;
 }
@@ -1047,10 +1049,13 @@ __global__ void k_fill(T *__restrict__ a, const int64_t n) {
     for (int64_t i = nv * V + g; i < n; i += stride) a[i] = T(0);
 }
 
-// Sec. 4.2.1: valsbar_i (+)= histbar[k_i] (0 for out-of-range keys).
+// Sec. 4.2.1: valsbar_i (+)= histbar[k_i] (0 for out-of-range keys); hist0bar in
+// the same launch.
 template <typename T>
 __global__ void k_hist_add_vjp(const int32_t *__restrict__ keys, const T *__restrict__ hb, T *__restrict__ vb,
-                               const int64_t n, const int64_t m, const int accumulate) {
+                               T *__restrict__ h0b, const int64_t n, const int64_t m, const int accumulate,
+                               unsigned *__restrict__ header) {
+    zero_header(header);
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t nv = n / 4;
@@ -1071,13 +1076,8 @@ __global__ void k_hist_add_vjp(const int32_t *__restrict__ keys, const T *__rest
         const T gv = in_range(k, m) ? hb[k] : T(0);
         vb[i] = accumulate ? vb[i] + gv : gv;
     }
-}
-
-// hist0bar (+)= histbar, masked per operator.
-template <typename T>
-__global__ void k_h0bar_add(const T *__restrict__ hb, T *__restrict__ h0b, const int64_t m, const int accumulate) {
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x)
-        h0b[j] = accumulate ? h0b[j] + hb[j] : hb[j];
+    if (h0b)  // hist0bar (+)= histbar
+        for (int64_t j = g; j < m; j += stride) h0b[j] = accumulate ? h0b[j] + hb[j] : hb[j];
 }
 
 // Fig. 5 return sweep: valsbar[is[j]] += histbar[j]; hist0bar[j] gets histbar[j] where hist0 won.
@@ -1391,6 +1391,7 @@ static Launch shape(adc_op op, size_t s, HistStrategy st, int64_t m, int64_t n) 
 }
 
 template <typename K> static bool set_smem(K kernel, size_t smem) {
+    if (smem <= 48 * 1024) return true;  // what every kernel may use
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess;
 }
 
@@ -1519,7 +1520,7 @@ static adc_status hist_primal_t(adc_op op, int64_t n, int64_t m, const int32_t *
             return part_fwd(kPPrimMul, dt, n, m, keys, vals, h0, hist, nullptr, nullptr, nullptr, ws,
                             part_off(op, dt, m), s);
         if (n == 0 || st == kGlobal) {
-            k_hist_init<T><<<gm, 256, 0, s>>>(hist, h0, m, T(1));
+            k_hist_init<T><<<gm, 256, 0, s>>>(hist, h0, m, T(1), nullptr);
             if (n > 0) k_prim_mul_global<T><<<gglob, 256, 0, s>>>(keys, vals, n, m, hist, err);
             return check_launch();
         }
@@ -1584,10 +1585,12 @@ static adc_status hist_fwd_t(adc_op op, int64_t n, int64_t m, const int32_t *key
     const unsigned gm = grid_for(m, 4);
     switch (op) {
     case ADC_OP_ADD: {
-        if (st == kPart && n > 0)
+        if (st == kPart && n > 0) {
+            if (cudaMemsetAsync(ws, 0, kWsHeader, s) != cudaSuccess) return ADC_ERR_CUDA;
             return part_fwd(kPAdd, dt_of<T>(), n, m, keys, vals, h0, hist, nullptr, nullptr, nullptr, ws,
                             part_off(op, dt_of<T>(), m), s);
-        k_hist_init<T><<<gm, 256, 0, s>>>(hist, h0, m, T(0));
+        }
+        k_hist_init<T><<<gm, 256, 0, s>>>(hist, h0, m, T(0), err);  // and the workspace's header
         if (n == 0) return check_launch();
         if (st == kGlobal) {
             k_hist_add_global<T><<<L.grid, L.block, 0, s>>>(keys, vals, n, m, hist);
@@ -1779,8 +1782,8 @@ static adc_status hist_vjp_t(adc_op op, int64_t n, int64_t m, const int32_t *key
     const unsigned gn8 = grid_for(n / 8 + 1, 8);  // the * vjp: 8 elements per step
     switch (op) {
     case ADC_OP_ADD:
-        if (n > 0) k_hist_add_vjp<T><<<gn, 256, 0, s>>>(keys, hb, vb, n, m, acc);
-        if (h0b) k_h0bar_add<T><<<gm, 256, 0, s>>>(hb, h0b, m, acc);
+        k_hist_add_vjp<T><<<h0b && gm > gn ? gm : gn, 256, 0, s>>>(keys, hb, vb, h0b, n, m, acc,
+                                                                   static_cast<unsigned *>(ws));
         return check_launch();
     case ADC_OP_MIN:
     case ADC_OP_MAX: {

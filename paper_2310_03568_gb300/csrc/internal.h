@@ -40,7 +40,8 @@ inline int arity(adc_op op) {
 }
 inline size_t elem_bytes(adc_op op, adc_dtype dt) { return (size_t)arity(op) * (dt == ADC_F64 ? 8 : 4); }
 
-// scan.cu
+// scan.cu (scan_fwd and scan_vjp zero the workspace's header themselves, with
+// their look-back words)
 size_t scan_ws_bytes(adc_op op, adc_dtype dt, int64_t n);
 adc_status scan_fwd(adc_op op, adc_dtype dt, int64_t n, const void *x, void *y, void *ws, cudaStream_t s);
 adc_status scan_vjp(adc_op op, adc_dtype dt, int64_t n, const void *x, const void *y, const void *ybar,

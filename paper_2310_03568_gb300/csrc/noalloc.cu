@@ -106,6 +106,5 @@ extern "C" adc_status adc_scan_fwd_noalloc(adc_op op, adc_dtype dt, int64_t n, c
     adc_status st = noalloc_scratch(&scratch);
     if (st != ADC_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (cudaMemsetAsync(scratch, 0, kWsHeader, s) != cudaSuccess) return ADC_ERR_CUDA;
     return scan_fwd(op, dt, n, x, y, scratch, s);
 }

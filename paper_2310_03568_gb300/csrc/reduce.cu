@@ -329,7 +329,9 @@ k_reduce_general_vjp(const Op op, const typename Op::State *__restrict__ x, cons
 
 // ------------------------------------------------------------- simple vjps --
 template <typename T>
-__global__ void k_vjp_add(T *__restrict__ xbar, const T *__restrict__ ybar, const int64_t n, const int accumulate) {
+__global__ void k_vjp_add(T *__restrict__ xbar, const T *__restrict__ ybar, const int64_t n, const int accumulate,
+                          unsigned *__restrict__ header) {
+    zero_header(header);
     const T yb = __ldg(ybar);
     constexpr int V = 16 / sizeof(T);
     const int64_t nv = n / V;
@@ -347,7 +349,8 @@ __global__ void k_vjp_add(T *__restrict__ xbar, const T *__restrict__ ybar, cons
 
 template <typename T>
 __global__ void k_vjp_sel_fill(T *__restrict__ xbar, const T *__restrict__ ybar, const int32_t *__restrict__ kp,
-                               const int64_t n) {
+                               const int64_t n, unsigned *__restrict__ header) {
+    zero_header(header);
     const T yb = __ldg(ybar);
     const int64_t kk = __ldg(kp);
     constexpr int V = 16 / sizeof(T);
@@ -374,7 +377,8 @@ __global__ void k_vjp_sel_acc(T *__restrict__ xbar, const T *__restrict__ ybar, 
 template <typename T>
 __global__ void k_vjp_mul(T *__restrict__ xbar, const T *__restrict__ x, const T *__restrict__ ybar,
                           const int32_t *__restrict__ n0p, const T *__restrict__ pp, const int64_t n,
-                          const int accumulate) {
+                          const int accumulate, unsigned *__restrict__ header) {
+    zero_header(header);
     const T yb = __ldg(ybar);
     const int32_t n0 = __ldg(n0p);
     const T p = __ldg(pp);
@@ -585,12 +589,16 @@ static unsigned elementwise_grid(int64_t work) {
 
 template <typename T>
 static adc_status red_vjp_t(adc_op op, int64_t n, const void *xv, const void *yv, const void *saved,
-                            const void *ybar, void *xbar, int acc, cudaStream_t s) {
+                            const void *ybar, void *xbar, int acc, void *ws, cudaStream_t s) {
+    unsigned *hdr = static_cast<unsigned *>(ws);
+    // the three kernels of +, min / max and * zero the header themselves
+    const bool own = op == ADC_OP_ADD || op == ADC_OP_MUL || ((op == ADC_OP_MIN || op == ADC_OP_MAX) && !acc);
+    if ((n == 0 || !own) && cudaMemsetAsync(ws, 0, kWsHeader, s) != cudaSuccess) return ADC_ERR_CUDA;
     if (n == 0) return ADC_OK;
     constexpr int V = 16 / sizeof(T);
     switch (op) {
     case ADC_OP_ADD:
-        k_vjp_add<T><<<elementwise_grid(n / V + 1), 256, 0, s>>>(static_cast<T *>(xbar), static_cast<const T *>(ybar), n, acc);
+        k_vjp_add<T><<<elementwise_grid(n / V + 1), 256, 0, s>>>(static_cast<T *>(xbar), static_cast<const T *>(ybar), n, acc, hdr);
         return check_launch();
     case ADC_OP_MIN:
     case ADC_OP_MAX:
@@ -599,13 +607,13 @@ static adc_status red_vjp_t(adc_op op, int64_t n, const void *xv, const void *yv
                                              static_cast<const int32_t *>(saved), n);
         else
             k_vjp_sel_fill<T><<<elementwise_grid(n / V + 1), 256, 0, s>>>(
-                static_cast<T *>(xbar), static_cast<const T *>(ybar), static_cast<const int32_t *>(saved), n);
+                static_cast<T *>(xbar), static_cast<const T *>(ybar), static_cast<const int32_t *>(saved), n, hdr);
         return check_launch();
     case ADC_OP_MUL:
         k_vjp_mul<T><<<elementwise_grid((n + V - 1) / V), 256, 0, s>>>(
             static_cast<T *>(xbar), static_cast<const T *>(xv), static_cast<const T *>(ybar),
             static_cast<const int32_t *>(saved), reinterpret_cast<const T *>(static_cast<const char *>(saved) + 8), n,
-            acc);
+            acc, hdr);
         return check_launch();
     case ADC_OP_SOP: {
         constexpr int PV = 16 / sizeof(Pair<T>) > 0 ? 16 / sizeof(Pair<T>) : 1;
@@ -658,9 +666,8 @@ static adc_status red_vjp_t(adc_op op, int64_t n, const void *xv, const void *yv
 
 adc_status reduce_vjp(adc_op op, adc_dtype dt, int64_t n, const void *x, const void *y, const void *saved,
                       const void *ybar, void *xbar, int accumulate, void *ws, cudaStream_t s) {
-    (void)ws;
-    return dt == ADC_F64 ? red_vjp_t<double>(op, n, x, y, saved, ybar, xbar, accumulate, s)
-                         : red_vjp_t<float>(op, n, x, y, saved, ybar, xbar, accumulate, s);
+    return dt == ADC_F64 ? red_vjp_t<double>(op, n, x, y, saved, ybar, xbar, accumulate, ws, s)
+                         : red_vjp_t<float>(op, n, x, y, saved, ybar, xbar, accumulate, ws, s);
 }
 
 }  // namespace adc

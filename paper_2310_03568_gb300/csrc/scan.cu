@@ -805,7 +805,7 @@ size_t scan_ws_bytes(adc_op op, adc_dtype dt, int64_t n) {
 
 template <class Op, int ITEMS, bool REVERSE>
 static adc_status launch(const Op &o, int64_t n, void *ws, cudaStream_t s) {
-    return run_scan<Op, ITEMS, REVERSE>(o, n, ws, 0, static_cast<char *>(ws) + kWsHeader, s);
+    return run_scan<Op, ITEMS, REVERSE>(o, n, ws, 0, static_cast<char *>(ws) + kWsHeader, s, ws);
 }
 // The streaming engine's shape per operator (n = 1e8 fp32, n = 1e7 fp64; the
 // figures are this shape's against the next best one measured).  One input
@@ -835,11 +835,12 @@ static adc_status launch_auto(const Op &o, int64_t n, void *ws, cudaStream_t s) 
                                                n * (int64_t)sizeof(typename Op::Elem) >= kStreamMinBytes);
     if (stream && stream_ready<Op, 8, P::kRow, P::kStages, P::kAhead, P::kSplit, REVERSE>())
         return run_scan_stream<Op, 8, P::kRow, P::kStages, P::kAhead, P::kSplit, REVERSE>(
-            o, n, ws, 0, static_cast<char *>(ws) + kWsHeader, ScanShape<Op, ITEMS>::region(n), s);
+            o, n, ws, ScanShape<Op, ITEMS>::region(n), s);
     return launch<Op, ITEMS, REVERSE>(o, n, ws, s);
 }
 template <class Op, int ITEMS, bool REVERSE>
 static adc_status launch_staged(const Op &o, int64_t n, void *ws, cudaStream_t s) {
+    if (cudaMemsetAsync(ws, 0, kWsHeader, s) != cudaSuccess) return ADC_ERR_CUDA;
     if (g_scan_engine == 4) return run_scan_tma<Op, ITEMS, REVERSE>(o, n, ws, 0, static_cast<char *>(ws) + kWsHeader, s);
     return run_scan_staged<Op, ITEMS, REVERSE>(o, n, ws, 0, static_cast<char *>(ws) + kWsHeader, s);
 }
@@ -1078,6 +1079,7 @@ static adc_status scan_fwd_t(adc_op op, int64_t n, const void *x, void *y, void 
 }
 
 adc_status scan_fwd(adc_op op, adc_dtype dt, int64_t n, const void *x, void *y, void *ws, cudaStream_t s) {
+    if (n == 0) return cudaMemsetAsync(ws, 0, kWsHeader, s) == cudaSuccess ? ADC_OK : ADC_ERR_CUDA;
     return dt == ADC_F64 ? scan_fwd_t<double>(op, n, x, y, ws, s) : scan_fwd_t<float>(op, n, x, y, ws, s);
 }
 
@@ -1184,6 +1186,7 @@ static adc_status scan_vjp_t(adc_op op, int64_t n, const void *x, const void *y,
 
 adc_status scan_vjp(adc_op op, adc_dtype dt, int64_t n, const void *x, const void *y, const void *ybar, void *xbar,
                     int accumulate, void *ws, cudaStream_t s) {
+    if (n == 0) return cudaMemsetAsync(ws, 0, kWsHeader, s) == cudaSuccess ? ADC_OK : ADC_ERR_CUDA;
     return dt == ADC_F64 ? scan_vjp_t<double>(op, n, x, y, ybar, xbar, accumulate, ws, s)
                          : scan_vjp_t<float>(op, n, x, y, ybar, xbar, accumulate, ws, s);
 }

@@ -710,14 +710,19 @@ extern int g_scan_range_tiles;
 
 // Queue one scan.  `ws` is the call's workspace (error word and counter slot
 // `slot` in its header); `region` holds this launch's tile flags and states.
+// `zero_from`: where the zeroing of the region starts -- the workspace itself
+// where its header lies directly before the region and is not zeroed yet (one
+// memset instead of two).
 template <class Op, int ITEMS, bool REVERSE>
-adc_status run_scan(const Op &op, int64_t n, void *ws, int slot, void *region, cudaStream_t s) {
+adc_status run_scan(const Op &op, int64_t n, void *ws, int slot, void *region, cudaStream_t s,
+                    void *zero_from = nullptr) {
     if (n == 0) return ADC_OK;
     using Sh = ScanShape<Op, ITEMS>;
     const int64_t T = Sh::tiles(n);
     const ScanWs L = scan_ws_layout(T, sizeof(typename Op::State));
     char *w = static_cast<char *>(region);
-    if (cudaMemsetAsync(w, 0, L.bytes, s) != cudaSuccess) return ADC_ERR_CUDA;
+    char *z = zero_from ? static_cast<char *>(zero_from) : w;
+    if (cudaMemsetAsync(z, 0, L.bytes + (size_t)(w - z), s) != cudaSuccess) return ADC_ERR_CUDA;
     const DevCtl ctl = make_ctl(ws, slot);
     if constexpr (per_tile_only<Op>(0)) {
         constexpr int TH = op_threads<Op>(0);

@@ -582,10 +582,10 @@ template <class Op, int NWC, int RB, int STAGES, int AHEAD, bool SPLIT, bool REV
 // modulo kStreamReps, so that fewer blocks poll the same lines.
 constexpr int kStreamReps = 4;
 
-// Queue one streaming scan (workspace and region as for run_scan; the region
-// has `avail` bytes, which bound the copies).
+// Queue one streaming scan of the whole call: the workspace's header, not zeroed
+// yet, and the region after it, whose `avail` bytes bound the copies.
 template <class Op, int NWC, int RB, int STAGES, int AHEAD, bool SPLIT, bool REVERSE>
-adc_status run_scan_stream(const Op &op, int64_t n, void *ws, int slot, void *region, size_t avail, cudaStream_t s) {
+adc_status run_scan_stream(const Op &op, int64_t n, void *ws, size_t avail, cudaStream_t s) {
     if (n == 0) return ADC_OK;
     using Sh = StreamShape<Op, NWC, RB, STAGES>;
     if (!stream_ready<Op, NWC, RB, STAGES, AHEAD, SPLIT, REVERSE>()) return ADC_ERR_CUDA;
@@ -593,10 +593,11 @@ adc_status run_scan_stream(const Op &op, int64_t n, void *ws, int slot, void *re
     const size_t one = (size_t)T * Tagged<typename Op::State>::K * 8;
     int reps = (int)(avail / one < (size_t)kStreamReps ? avail / one : (size_t)kStreamReps);
     if (reps < 1) return ADC_ERR_WORKSPACE;
-    if (cudaMemsetAsync(region, 0, one * reps, s) != cudaSuccess) return ADC_ERR_CUDA;
+    void *region = static_cast<char *>(ws) + kWsHeader;
+    if (cudaMemsetAsync(ws, 0, kWsHeader + one * reps, s) != cudaSuccess) return ADC_ERR_CUDA;
     const int64_t G = num_sms();
     k_scan_stream<Op, NWC, RB, STAGES, AHEAD, SPLIT, REVERSE><<<(unsigned)(T < G ? T : G), stream_threads(NWC, SPLIT), Sh::kSmem, s>>>(
-        op, n, T, static_cast<unsigned long long *>(region), reps, make_ctl(ws, slot));
+        op, n, T, static_cast<unsigned long long *>(region), reps, make_ctl(ws, 0));
     return check_launch();
 }
 

@@ -224,11 +224,7 @@ size_t tscan_ws_bytes(int k, const adc_op *ops, adc_dtype dt, int64_t n, bool ro
     return tlayout(k, ops, dt, n, rows).bytes;
 }
 
-static char *block_ws(char *ws, const TLayout &L, int c, cudaStream_t s, bool *ok) {
-    char *w = ws + L.blocks + (size_t)c * L.stride;
-    *ok = cudaMemsetAsync(w, 0, kWsHeader, s) == cudaSuccess;
-    return w;
-}
+static char *block_ws(char *ws, const TLayout &L, int c) { return ws + L.blocks + (size_t)c * L.stride; }
 
 static adc_status gather_errors(char *ws, const TLayout &L, int k, cudaStream_t s) {
     k_tuple_errors<<<1, 64, 0, s>>>(reinterpret_cast<unsigned *>(ws), ws + L.blocks, k, L.stride);
@@ -239,9 +235,7 @@ static adc_status gather_errors(char *ws, const TLayout &L, int k, cudaStream_t 
 static adc_status fwd_blocks(int k, const adc_op *ops, adc_dtype dt, int64_t n, const void *const *x, void *const *y,
                              char *ws, const TLayout &L, cudaStream_t s) {
     for (int c = 0; c < k; ++c) {
-        bool ok;
-        char *w = block_ws(ws, L, c, s, &ok);
-        if (!ok) return ADC_ERR_CUDA;
+        char *w = block_ws(ws, L, c);
         const adc_status st = scan_fwd(ops[c], dt, n, x[c], y[c], w, s);
         if (st != ADC_OK) return st;
     }
@@ -252,9 +246,7 @@ static adc_status vjp_blocks(int k, const adc_op *ops, adc_dtype dt, int64_t n, 
                              const void *const *y, const void *const *ybar, void *const *xbar, int acc, char *ws,
                              const TLayout &L, cudaStream_t s) {
     for (int c = 0; c < k; ++c) {
-        bool ok;
-        char *w = block_ws(ws, L, c, s, &ok);
-        if (!ok) return ADC_ERR_CUDA;
+        char *w = block_ws(ws, L, c);
         const adc_status st = scan_vjp(ops[c], dt, n, x[c], y[c], ybar[c], xbar[c], acc, w, s);
         if (st != ADC_OK) return st;
     }
