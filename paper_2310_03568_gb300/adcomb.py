@@ -13,6 +13,7 @@ saved-buffer queries).  Tensors are CUDA tensors; tuple operators take
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 import threading
 
@@ -42,6 +43,8 @@ _lib = None
 def lib():
     """Load libadcomb.so (build it first with paper_2310_03568_gb300.build.build())."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(LIB_PATH):
@@ -97,8 +100,10 @@ def _ptr(t):
 
 
 def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    # the handle of torch.cuda.current_stream(), without building a Stream object
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _check(fn, code):
@@ -149,10 +154,27 @@ def _n(x, op):
     return x.shape[0] if x.dim() > 0 else 1
 
 
-def _ws(kind, op, x, n, m, ws):
-    need = workspace_bytes(kind, op, x.dtype, n, m)
-    w = (ws or default_workspace(x.device)).get(need, x.device)
-    return w, w.numel()
+def _with_ws(fn, ws, device, need, call):
+    """call(pointer, bytes) with a workspace: the one at hand first, and only when the library says that it is
+    too small (before it queues anything) is the size asked for and the workspace grown."""
+    w = ws or default_workspace(device)
+    buf = w.buf
+    code = 3
+    if buf is not None and buf.device == device:
+        code = call(buf.data_ptr(), buf.numel())
+    if code == 3:
+        buf = w.get(need(), device)
+        code = call(buf.data_ptr(), buf.numel())
+    _check(fn, code)
+
+
+def _saved(kind, op, dtype, n, m, device):
+    # lin's residuals depend on the sort path chosen; the others' sizes on the arguments alone
+    size = saved_bytes(kind, op, dtype, n, m) if op == "lin" else _saved_size(kind, op, dtype, n, m)
+    return torch.empty(max(size, 16), dtype=torch.uint8, device=device)
+
+
+_saved_size = functools.lru_cache(maxsize=256)(saved_bytes)
 
 
 # ---------------------------------------------------------------- reduce ----
@@ -163,10 +185,10 @@ def reduce_fwd(op, x, y=None, saved=None, ws=None, stream=None):
     if y is None:
         y = torch.empty((d,) if d > 1 else (1,), dtype=x.dtype, device=x.device)
     if saved is None:
-        saved = torch.empty(max(saved_bytes("reduce", op, x.dtype, n), 16), dtype=torch.uint8, device=x.device)
-    w, wb = _ws("reduce", op, x, n, 0, ws)
-    _check("adc_reduce_fwd", lib().adc_reduce_fwd(OPS[op], _dt(x), n, _ptr(x), _ptr(y), _ptr(saved), _ptr(w), wb,
-                                                   _stream(stream)))
+        saved = _saved("reduce", op, x.dtype, n, 0, x.device)
+    _with_ws("adc_reduce_fwd", ws, x.device, lambda: workspace_bytes("reduce", op, x.dtype, n),
+             lambda w, wb: lib().adc_reduce_fwd(OPS[op], _dt(x), n, _ptr(x), _ptr(y), _ptr(saved), w, wb,
+                                                _stream(stream)))
     return y, saved
 
 
@@ -174,9 +196,9 @@ def reduce_vjp(op, x, y, saved, ybar, xbar=None, accumulate=False, ws=None, stre
     n = x.shape[0]
     if xbar is None:
         xbar = torch.empty_like(x)
-    w, wb = _ws("reduce", op, x, n, 0, ws)
-    _check("adc_reduce_vjp", lib().adc_reduce_vjp(OPS[op], _dt(x), n, _ptr(x), _ptr(y), _ptr(saved), _ptr(ybar),
-                                                   _ptr(xbar), int(bool(accumulate)), _ptr(w), wb, _stream(stream)))
+    _with_ws("adc_reduce_vjp", ws, x.device, lambda: workspace_bytes("reduce", op, x.dtype, n),
+             lambda w, wb: lib().adc_reduce_vjp(OPS[op], _dt(x), n, _ptr(x), _ptr(y), _ptr(saved), _ptr(ybar),
+                                                _ptr(xbar), int(bool(accumulate)), w, wb, _stream(stream)))
     return xbar
 
 
@@ -185,8 +207,8 @@ def scan_fwd(op, x, y=None, ws=None, stream=None):
     n = x.shape[0]
     if y is None:
         y = torch.empty_like(x)
-    w, wb = _ws("scan", op, x, n, 0, ws)
-    _check("adc_scan_fwd", lib().adc_scan_fwd(OPS[op], _dt(x), n, _ptr(x), _ptr(y), _ptr(w), wb, _stream(stream)))
+    _with_ws("adc_scan_fwd", ws, x.device, lambda: workspace_bytes("scan", op, x.dtype, n),
+             lambda w, wb: lib().adc_scan_fwd(OPS[op], _dt(x), n, _ptr(x), _ptr(y), w, wb, _stream(stream)))
     return y
 
 
@@ -204,9 +226,9 @@ def scan_vjp(op, x, y, ybar, xbar=None, accumulate=False, ws=None, stream=None):
     n = ybar.shape[0]
     if xbar is None:
         xbar = torch.empty_like(ybar)
-    w, wb = _ws("scan", op, ybar, n, 0, ws)
-    _check("adc_scan_vjp", lib().adc_scan_vjp(OPS[op], _dt(ybar), n, _ptr(x), _ptr(y), _ptr(ybar), _ptr(xbar),
-                                               int(bool(accumulate)), _ptr(w), wb, _stream(stream)))
+    _with_ws("adc_scan_vjp", ws, ybar.device, lambda: workspace_bytes("scan", op, ybar.dtype, n),
+             lambda w, wb: lib().adc_scan_vjp(OPS[op], _dt(ybar), n, _ptr(x), _ptr(y), _ptr(ybar), _ptr(xbar),
+                                              int(bool(accumulate)), w, wb, _stream(stream)))
     return xbar
 
 
@@ -218,11 +240,10 @@ def hist_fwd(op, m, keys, vals, hist0=None, hist=None, saved=None, ws=None, stre
     if hist is None:
         hist = torch.empty((m, d) if d > 1 else (m,), dtype=vals.dtype, device=vals.device)
     if saved is None:
-        saved = torch.empty(max(saved_bytes("hist", op, vals.dtype, n, m), 16), dtype=torch.uint8,
-                            device=vals.device)
-    w, wb = _ws("hist", op, vals, n, m, ws)
-    _check("adc_hist_fwd", lib().adc_hist_fwd(OPS[op], _dt(vals), n, int(m), _ptr(keys), _ptr(vals), _ptr(hist0),
-                                               _ptr(hist), _ptr(saved), _ptr(w), wb, _stream(stream)))
+        saved = _saved("hist", op, vals.dtype, n, int(m), vals.device)
+    _with_ws("adc_hist_fwd", ws, vals.device, lambda: workspace_bytes("hist", op, vals.dtype, n, m),
+             lambda w, wb: lib().adc_hist_fwd(OPS[op], _dt(vals), n, int(m), _ptr(keys), _ptr(vals), _ptr(hist0),
+                                              _ptr(hist), _ptr(saved), w, wb, _stream(stream)))
     return hist, saved
 
 
@@ -232,9 +253,9 @@ def hist_primal(op, m, keys, vals, hist0=None, hist=None, ws=None, stream=None):
     d = ARITY[op]
     if hist is None:
         hist = torch.empty((m, d) if d > 1 else (m,), dtype=vals.dtype, device=vals.device)
-    w, wb = _ws("hist", op, vals, n, m, ws)
-    _check("adc_hist_fwd", lib().adc_hist_fwd(OPS[op], _dt(vals), n, int(m), _ptr(keys), _ptr(vals), _ptr(hist0),
-                                               _ptr(hist), None, _ptr(w), wb, _stream(stream)))
+    _with_ws("adc_hist_fwd", ws, vals.device, lambda: workspace_bytes("hist", op, vals.dtype, n, m),
+             lambda w, wb: lib().adc_hist_fwd(OPS[op], _dt(vals), n, int(m), _ptr(keys), _ptr(vals), _ptr(hist0),
+                                              _ptr(hist), None, w, wb, _stream(stream)))
     return hist
 
 
@@ -246,10 +267,10 @@ def hist_vjp(op, m, keys, vals, hist0, hist, saved, histbar, valsbar=None, hist0
         valsbar = torch.empty_like(vals)
     if hist0bar is None and want_hist0bar:
         hist0bar = torch.empty_like(histbar)
-    w, wb = _ws("hist", op, histbar, n, m, ws)
-    _check("adc_hist_vjp", lib().adc_hist_vjp(OPS[op], _dt(histbar), n, int(m), _ptr(keys), _ptr(vals), _ptr(hist0),
-                                               _ptr(hist), _ptr(saved), _ptr(histbar), _ptr(valsbar), _ptr(hist0bar),
-                                               int(bool(accumulate)), _ptr(w), wb, _stream(stream)))
+    _with_ws("adc_hist_vjp", ws, histbar.device, lambda: workspace_bytes("hist", op, histbar.dtype, n, m),
+             lambda w, wb: lib().adc_hist_vjp(OPS[op], _dt(histbar), n, int(m), _ptr(keys), _ptr(vals), _ptr(hist0),
+                                              _ptr(hist), _ptr(saved), _ptr(histbar), _ptr(valsbar), _ptr(hist0bar),
+                                              int(bool(accumulate)), w, wb, _stream(stream)))
     return valsbar, hist0bar
 
 

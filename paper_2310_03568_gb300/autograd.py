@@ -31,7 +31,8 @@ __all__ = ["reduce", "scan", "reduce_by_index", "ReduceFn", "ScanFn", "HistFn"]
 
 
 def _flat(x, d):
-    return x.contiguous() if d > 1 else x.contiguous().reshape(-1)
+    x = x.contiguous()
+    return x if d > 1 or x.dim() == 1 else x.reshape(-1)
 
 
 class ReduceFn(torch.autograd.Function):
