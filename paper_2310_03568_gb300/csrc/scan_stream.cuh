@@ -21,9 +21,9 @@
 //             runs.
 // What bounds it: the time from a tile's fold to its prefix, about 4 us at full
 // bandwidth, during which its inputs wait in shared memory.  With one input
-// array six 32 KB stages cover it (n = 1e8 fp32 + forward 0.138 ms, 0.85 of the
+// array six 32 KB stages cover it (n = 1e8 fp32 + forward 0.136 ms, 0.87 of the
 // 6.8 TB/s copy rate; the range engine, which reads the input twice, 0.215);
-// with three arrays four 48 KB stages do not (lin vjp 0.617 ms, 0.76; 0.764).
+// with three arrays four 48 KB stages do not (lin vjp 0.612 ms, 0.77; 0.764).
 // Hence: four copies of the aggregates, so that fewer blocks poll the same
 // lines (lin vjp 0.90 -> 0.72 ms before the roles were split); claims at the
 // pace of the folds (claimed in bursts, a block folds neighbouring tiles a
@@ -161,13 +161,13 @@ __device__ __forceinline__ void copy16(unsigned char *dst, const E *src, int64_t
 // 0.160 ms, n = 1e8 +): it lengthens the one chain that everything waits for.
 template <class Op, typename S>
 __device__ __forceinline__ bool stream_lookback(const Op &op, const unsigned long long *__restrict__ aggw,
-                                                int64_t stride, long long from, long long to, S *run,
+                                                unsigned stride, unsigned from, unsigned to, S *run,
                                                 long long limit) {
     constexpr int K = Tagged<S>::K;
     constexpr int Q = 5;  // 160 tiles: one per SM, so one step as a rule
     constexpr bool kLaneMajor = K > 4 || sizeof(typename Op::Scalar) == 8;
-    const int lane = threadIdx.x & 31;
-    for (long long base = from; base < to; base += 32 * Q) {
+    const unsigned lane = threadIdx.x & 31;
+    for (unsigned base = from; base < to; base += 32 * Q) {
         unsigned long long w[Q][K];
         unsigned todo = 0;
         const auto tile = [&](int q) { return base + (kLaneMajor ? lane * Q + q : 32 * q + lane); };
@@ -180,7 +180,7 @@ __device__ __forceinline__ bool stream_lookback(const Op &op, const unsigned lon
             for (int q = 0; q < Q; ++q)
                 if ((todo >> q) & 1u) {
 #pragma unroll
-                    for (int k = 0; k < K; ++k) w[q][k] = ld_relaxed_u64(aggw + k * stride + tile(q));
+                    for (int k = 0; k < K; ++k) w[q][k] = ld_relaxed_u64(aggw + (size_t)k * stride + tile(q));
                 }
 #pragma unroll
             for (int q = 0; q < Q; ++q)
@@ -239,10 +239,12 @@ k_scan_stream(const Op op, const int64_t n, const int64_t num_tiles, unsigned lo
     __shared__ __align__(8) unsigned long long s_bar_agg[STAGES], s_bar_pre[STAGES], s_bar_free[STAGES],
         s_bar_claim[RING];
     __shared__ S s_agg[STAGES][NWC], s_wex[STAGES][NWC], s_pre[STAGES];
-    __shared__ long long s_tile[RING];
+    __shared__ unsigned s_tile[RING];
     __shared__ volatile int s_abort;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const long long T_ = num_tiles;
+    // Tiles and slots are 32-bit: the rings' quotients and remainders are in every
+    // role's serial path, the look-back's above all.
+    const unsigned T_ = (unsigned)num_tiles;
     // the waits on other blocks (ctl.spin_limit) end before those inside the block
     const long long wait_limit = ctl.spin_limit < (1ll << 40) ? ctl.spin_limit * 16 : ctl.spin_limit;
     if (threadIdx.x == 0) {
@@ -258,9 +260,9 @@ k_scan_stream(const Op op, const int64_t n, const int64_t num_tiles, unsigned lo
     __syncthreads();
     // A whole warp's wait inside the block for use `slot` of a ring of barriers;
     // false, alike in every lane, if the block gave up or the limit ran out.
-    const auto wait_ring = [&](unsigned long long *bars, long long slot, int ring) -> bool {
+    const auto wait_ring = [&](unsigned long long *bars, unsigned slot, unsigned ring) -> bool {
         unsigned long long *bar = bars + slot % ring;
-        const unsigned parity = (unsigned)(slot / ring) & 1u;
+        const unsigned parity = (slot / ring) & 1u;
         bool ok = false;
         for (long long it = 0; it <= wait_limit && !s_abort; ++it)
             if ((ok = mbar_try_wait(bar, parity))) break;
@@ -273,12 +275,12 @@ k_scan_stream(const Op op, const int64_t n, const int64_t num_tiles, unsigned lo
 
     constexpr int kWorkers = SPLIT ? 2 * NWC : NWC;
     if (warp == kWorkers + 1) {  // -------------------------------------- look-back --
-        const unsigned long long *mine = aggw + (int64_t)(blockIdx.x % reps) * T_ * K;
+        const unsigned long long *mine = aggw + (size_t)(blockIdx.x % reps) * T_ * K;
         S run = op.identity();  // the exclusive prefix of tile `from`
-        long long from = 0;
-        for (long long i = 0;; ++i) {
+        unsigned from = 0;
+        for (unsigned i = 0;; ++i) {
             if (!wait_ring(s_bar_claim, i, RING)) return;
-            const long long t = s_tile[i % RING];
+            const unsigned t = s_tile[i % RING];
             if (t >= T_) return;
             const bool ok = stream_lookback(op, mine, T_, from, t, &run, ctl.spin_limit);
             if (!ok && lane == 0) give_up();
@@ -295,7 +297,7 @@ k_scan_stream(const Op op, const int64_t n, const int64_t num_tiles, unsigned lo
         // Tiles are claimed at the pace of the folds: claims in bursts would give a
         // block neighbouring tiles that it folds a whole round apart, and every
         // tile behind them would wait for that round.
-        const auto claimed = [&](long long slot, unsigned t) {  // lane 0
+        const auto claimed = [&](unsigned slot, unsigned t) {  // lane 0
             s_tile[slot % RING] = t;
             mbar_arrive(&s_bar_claim[slot % RING]);
         };
@@ -304,17 +306,17 @@ k_scan_stream(const Op op, const int64_t n, const int64_t num_tiles, unsigned lo
             for (int j = 0; j <= AHEAD; ++j) claimed(j, atomicAdd(ctl.counter, 1u));
             next = atomicAdd(ctl.counter, 1u);
         }
-        for (long long i = 0;; ++i) {
+        for (unsigned i = 0;; ++i) {
             if (!wait_ring(s_bar_claim, i, RING)) return;
-            const long long t = s_tile[i % RING];
+            const unsigned t = s_tile[i % RING];
             if (t >= T_ || !wait_ring(s_bar_agg, i, STAGES)) return;
             const S inc = warp_inclusive_scan(op, lane < NWC ? s_agg[i % STAGES][lane] : op.identity());
             const S total = shfl_idx(inc, NWC - 1);
-            if (lane < reps && t != ctl.stall_tile) {
+            if (lane < reps && (long long)t != ctl.stall_tile) {
                 const unsigned *w = reinterpret_cast<const unsigned *>(&total);
 #pragma unroll
                 for (int k = 0; k < K; ++k)
-                    st_relaxed_u64(aggw + ((int64_t)lane * K + k) * T_ + t, ((unsigned long long)kFlagAgg << 32) | w[k]);
+                    st_relaxed_u64(aggw + ((size_t)lane * K + k) * T_ + t, ((unsigned long long)kFlagAgg << 32) | w[k]);
             }
             S wex = shfl_up(inc, 1);
             if (lane == 0) wex = op.identity();
@@ -337,22 +339,22 @@ k_scan_stream(const Op op, const int64_t n, const int64_t num_tiles, unsigned lo
     const int seg = REVERSE ? NWC - 1 - w : w;  // the warp's segment of the tile, its lanes' rows
     const int row = REVERSE ? 31 - lane : lane;
     const int64_t nb = n * (int64_t)sizeof(E);
-    const auto segment = [&](long long slot, int s) -> Seg {
-        return Seg{smem_raw + (size_t)(slot % STAGES) * Sh::kData + (size_t)(w * Sh::NS + s) * Sh::SEGP};
+    const auto segment = [&](unsigned slot, int s) -> Seg {
+        return Seg{smem_raw + (slot % STAGES) * (unsigned)Sh::kData + (unsigned)(w * Sh::NS + s) * Sh::SEGP};
     };
     S *const s_ex = reinterpret_cast<S *>(smem_raw + STAGES * Sh::kData) + w * 32 + lane;  // + stage * NWC * 32
-    const auto first_byte = [&](long long t) -> int64_t {
+    const auto first_byte = [&](unsigned t) -> int64_t {
         const int64_t p = REVERSE ? T_ - 1 - t : t;
         return (p * NWC + seg) * (int64_t)Sh::SEG;
     };
 
     bool alive = true;
-    const auto load = [&](long long slot) {
+    const auto load = [&](unsigned slot) {
         if (!wait_ring(s_bar_claim, slot, RING)) {
             alive = false;
             return;
         }
-        const long long t = s_tile[slot % RING];
+        const unsigned t = s_tile[slot % RING];
         if (t < T_) {
             if (SPLIT && slot >= STAGES && !wait_ring(s_bar_free, slot - STAGES, STAGES)) {
                 alive = false;
@@ -389,7 +391,7 @@ k_scan_stream(const Op op, const int64_t n, const int64_t num_tiles, unsigned lo
         }
         cp_async_commit();
     };
-    const auto fold = [&](long long i, long long t) {
+    const auto fold = [&](unsigned i, unsigned t) {
         cp_async_wait<AHEAD - 1>();
         __syncwarp();
         const int64_t e0 = first_byte(t) / (int64_t)sizeof(E) + (int64_t)row * Sh::EPR;
@@ -429,7 +431,7 @@ k_scan_stream(const Op op, const int64_t n, const int64_t num_tiles, unsigned lo
         __syncwarp();
         if (lane == kWarp - 1) mbar_arrive(&s_bar_agg[i % STAGES]);
     };
-    const auto store = [&](long long j) {
+    const auto store = [&](unsigned j) {
         S run = op.combine(op.combine(s_pre[j % STAGES], s_wex[j % STAGES][w]), s_ex[(j % STAGES) * NWC * 32]);
         const int64_t b0 = first_byte(s_tile[j % RING]);
         const int64_t e0 = b0 / (int64_t)sizeof(E) + (int64_t)row * Sh::EPR;
@@ -518,7 +520,7 @@ k_scan_stream(const Op op, const int64_t n, const int64_t num_tiles, unsigned lo
     };
 
     if (SPLIT && warp >= NWC) {
-        for (long long j = 0;; ++j) {
+        for (unsigned j = 0;; ++j) {
             if (!wait_ring(s_bar_claim, j, RING)) return;
             if (s_tile[j % RING] >= T_) return;
             if (!wait_ring(s_bar_pre, j, STAGES)) {
@@ -530,18 +532,18 @@ k_scan_stream(const Op op, const int64_t n, const int64_t num_tiles, unsigned lo
         }
     }
     for (int j = 0; j < AHEAD && alive; ++j) load(j);
-    constexpr int D = STAGES - AHEAD;
-    long long end = -1;  // first slot without a tile
-    for (long long i = 0; alive; ++i) {
-        if (end < 0) {
-            const long long t = s_tile[i % RING];
+    constexpr unsigned D = STAGES - AHEAD, kNone = 0xffffffffu;
+    unsigned end = kNone;  // first slot without a tile
+    for (unsigned i = 0; alive; ++i) {
+        if (end == kNone) {
+            const unsigned t = s_tile[i % RING];
             if (t >= T_) end = i;
             else fold(i, t);
         }
         if constexpr (SPLIT) {
-            if (end >= 0) break;
+            if (end != kNone) break;
         } else {
-            if (end >= 0 && i - D >= end) break;
+            if (end != kNone && i >= D && i - D >= end) break;
             if (i >= D) {
                 if (!wait_ring(s_bar_pre, i - D, STAGES)) {
                     alive = false;
@@ -550,7 +552,7 @@ k_scan_stream(const Op op, const int64_t n, const int64_t num_tiles, unsigned lo
                 store(i - D);
             }
         }
-        if (end < 0) load(i + AHEAD);
+        if (end == kNone) load(i + AHEAD);
     }
     cp_async_wait<0>();
     if (!alive && lane == 0) give_up();
