@@ -279,8 +279,9 @@ size_t adc_batched_workspace_bytes(int32_t count, int64_t total_bins);
  * instances the selected element's index within the instance, n when the zero
  * initial value won or the bin is empty; unused for ADD), loss_parts (fp32,
  * [count]) and loss (fp32, one value).  desc and items are DEVICE copies.
- * smem_bins: shared-memory table size per block in bins (the instances with
- * more bins use global atomics); 0 picks the default.
+ * smem_bins: shared-memory table size per block in bins of a MAX instance (8
+ * bytes; an ADD instance's bins take 4; the instances with more bins use global
+ * atomics); 0 picks the default.
  */
 adc_status adc_batched_hist_scan_fwd(const adc_instance *desc, int32_t count, const adc_work *items,
                                      int64_t n_items, int64_t total_bins, const int32_t *keys,
@@ -441,7 +442,7 @@ void adc_debug_set_scan_prefetch(int on);
 
 /*
  * Tuning hook: elements per thread and step of the batched histogram launch
- * (1, 4 or 8; anything else selects the default, 4).  A step's key and value
+ * (1, 4 or 8; anything else selects the default, 8).  A step's key and value
  * loads are all issued before its atomic updates.  Results do not depend on it
  * beyond the order of the + atomics.
  */

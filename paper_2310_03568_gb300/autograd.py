@@ -16,8 +16,8 @@ Residual policy (``policy="save"`` or ``"recompute"``):
                    more pass).
   reduce_by_index +: keys; min/max: keys and is[m]; *: keys, values, (n0, p);
           lin    : m <= 2047: per (bin, input chunk) prefix and suffix tables
-                   (about 16*m*n/4096 bytes; the chunk-local sort is redone in
-                   backward anyway); larger m: the stable permutation with the
+                   (about 16*m*n/4096 bytes; the walks over the chunks are
+                   redone in backward anyway); larger m: the stable permutation with the
                    sorted keys and values (16 B/element).  "recompute" re-runs
                    the forward in backward instead.
 """

@@ -6,7 +6,8 @@
 //   scan_i  = scan (+) hist_i                                        (Sec. 5.1)
 //   loss    = sum_i sum_j scan_i[j]                                  (Sec. 3)
 // vjp: ybar of the sum is a broadcast (Sec. 3.2.1), the +-scan's adjoint a
-// reverse +-scan (Sec. 5.3.1), then the gather of Sec. 4.2.1 (ADD) or the
+// reverse +-scan (Sec. 5.3.1) -- of a constant, so (m - j) lossbar without a
+// pass over memory -- then the gather of Sec. 4.2.1 (ADD) or the
 // argmax scatter of Fig. 5 (MAX; the zero initial value wins ties).
 //
 // Launches: init (one block per instance) -> histogram (persistent blocks
@@ -14,9 +15,8 @@
 // shared-memory table when the instance's bins fit and the item is long
 // enough to amortise it, global atomics otherwise) -> scan + loss (one block
 // per instance, deterministic loss from per-instance partials combined in
-// instance order by the last block).  Backward: reverse scan of the loss
-// adjoint per instance -> per-item gather / zero-fill -> per-instance argmax
-// scatter.
+// instance order by the last block).  Backward: per-item gather / zero-fill ->
+// per-instance histogram adjoints and argmax scatter.
 #include <algorithm>
 #include <vector>
 

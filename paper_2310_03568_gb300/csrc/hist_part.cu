@@ -9,15 +9,15 @@
 // L2 latency with DRAM nearly idle.  Here the bins are split into B buckets of
 // W consecutive bins, W chosen so that one bucket's table fills one block's
 // shared memory, and the elements are moved by bucket into scratch:
-//   1. count   per chunk of kPartChunk elements, how many fall in each bucket;
-//   2. scan    exclusive +-scan of the bucket-major count matrix: where each
-//              (bucket, chunk) run starts (the look-back scan engine);
-//   3. scatter each chunk is counting-sorted by bucket in shared memory and
-//              written out as contiguous runs of (bin within the bucket, 16
-//              bits; payload), the payload being the value (+, *) or the packed
-//              (value, index) key (lifted min/max); for fp32 a persistent block
-//              per SM with the chunks staged by bulk (TMA) copies one ahead;
-//   4. table   one block per bucket streams its run into a shared-memory table
+//   1. count   how many elements fall in each bucket; the last block to finish
+//              turns the totals into the buckets' starts and cursors;
+//   2. scatter each chunk of kPartChunk elements is counting-sorted by bucket
+//              in shared memory and written out as contiguous runs of (bin
+//              within the bucket, 16 bits; payload) at places reserved at the
+//              buckets' cursors, the payload being the value (+, *) or the
+//              packed (value, index) key (lifted min/max); for fp32 two
+//              persistent blocks per SM, chunks staged by bulk (TMA) copies;
+//   3. table   one block per bucket streams its run into a shared-memory table
 //              of W bins and writes them out.  Every bin belongs to exactly one
 //              bucket, so there are no global atomics at all.
 // Traffic per element, fp32 *: 4 (count) + 8 + 6 (scatter) + 6 (table) bytes,
@@ -308,7 +308,7 @@ k_part_count(const int32_t *__restrict__ keys, const int64_t n, const int64_t m,
     if (tid == kPartThreads - 1 && B == kPartMaxBuckets) start[B] = run;
 }
 
-// 3. Counting sort of one chunk by bucket in shared memory, then contiguous
+// 2. Counting sort of one chunk by bucket in shared memory, then contiguous
 // runs out: obin = bin - bucket * W, oval = payload, in the run that the chunk
 // reserves at its bucket's cursor.
 // Register-lean so that two blocks fit an SM: a thread keeps only each
@@ -571,7 +571,7 @@ k_part_scatter_tma(const int32_t *__restrict__ keys, const float *__restrict__ v
     }
 }
 
-// 4. One block per bucket: the bucket's W bins in shared memory, its run of
+// 3. One block per bucket: the bucket's W bins in shared memory, its run of
 // (bin, payload) streamed in, the bins written out.
 template <typename T, int MODE>
 __global__ void __launch_bounds__(kPartTableThreads)

@@ -73,10 +73,6 @@ adc_status histgen_vjp(adc_dtype dt, int64_t n, int64_t m, const int32_t *keys, 
                        const void *hist0, const void *hist, const void *saved, const void *histbar,
                        void *valsbar, void *hist0bar, int accumulate, void *ws, cudaStream_t s);
 
-size_t excl_scan_i32_region(int64_t n);
-adc_status excl_scan_i32(const int32_t *in, int32_t *out, int64_t n, void *ws, int slot, void *region,
-                         cudaStream_t s);
-
 // hist_lin.cu (general reduce_by_index, linFnComp, m <= 2047 fp32 / 1023 fp64:
 // hierarchical stable sort)
 bool linh_applicable(adc_dtype dt, int64_t m);
