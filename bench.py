@@ -50,14 +50,14 @@ def launches(phase, op, m, n):
     forward is init + table kernel + finaliser (for * with per-thread or
     per-warp tables: table kernel + cross-block reduce, which finalises; for
     min/max in two passes: value rows + row reduce + index pass + decode), or,
-    partitioned by bin range (m >= 2^18), count + count scan + scatter +
-    per-bucket tables (which also finalise);
+    partitioned by bin range (m >= 2^18), count + scatter + per-bucket tables
+    (which also finalise);
     the * vjp is coefficient tables + gather; the min/max vjp is a zero-fill +
     scatter, or, when bins are sparse (8m > n), a bitmap of the selected
     elements + one streaming pass."""
     if phase == "fwd":
         if m >= (1 << 18):
-            return 4
+            return 3
         # * with per-thread or per-warp tables: table kernel + cross-block reduce
         if op == "mul":
             return 2 if m * 8 * 8 <= 48 * 1024 else 3
