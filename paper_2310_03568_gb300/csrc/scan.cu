@@ -122,6 +122,8 @@ template <typename T, int ITEMS> struct FwdAdd : PlainScan<T, ITEMS, FwdAdd<T, I
     static constexpr bool kKeepPrefix = sizeof(T) == 8;  // fp64: the combine is the bound
     __device__ T identity() const { return T(0); }
     __device__ T combine(T a, T b) const { return a + b; }
+    static constexpr int kExact = sizeof(T) == 4 ? kExactSum : kExactNone;
+    __device__ void extend(T &hi, T &lo, T d) const { add_carry(hi, lo, d); }
 };
 
 template <typename T, int ITEMS> struct FwdMul : PlainScan<T, ITEMS, FwdMul<T, ITEMS>> {
@@ -129,6 +131,9 @@ template <typename T, int ITEMS> struct FwdMul : PlainScan<T, ITEMS, FwdMul<T, I
     static constexpr bool kKeepPrefix = sizeof(T) == 8;  // fp64: the combine is the bound
     __device__ T identity() const { return T(1); }
     __device__ T combine(T a, T b) const { return a * b; }
+    static constexpr int kExact = sizeof(T) == 4 ? kExactProduct : kExactNone;
+    __device__ static T &coef(T &s) { return s; }
+    __device__ static const T &coef(const T &s) { return s; }
 };
 
 // min / max scans: the running extremum; the earlier operand wins ties (the
@@ -161,6 +166,9 @@ template <typename T, int ITEMS> struct FwdLin : PlainScan<Pair<T>, ITEMS, FwdLi
     static constexpr bool kKeepPrefix = sizeof(T) == 8;  // fp64: the combine is the bound
     __device__ Pair<T> identity() const { return {T(0), T(1)}; }
     __device__ Pair<T> combine(const Pair<T> &a, const Pair<T> &b) const { return {b.b + b.c * a.b, b.c * a.c}; }
+    static constexpr int kExact = sizeof(T) == 4 ? kExactProduct : kExactNone;
+    __device__ static T &coef(Pair<T> &s) { return s.c; }
+    __device__ static const T &coef(const Pair<T> &s) { return s.c; }
 };
 
 // sumOfProd (Fig. 8): (p1,s1) . (p2,s2) = (p1 + p2 + s1*s2, s1 + s2)
@@ -170,6 +178,14 @@ template <typename T, int ITEMS> struct FwdSop : PlainScan<Pair<T>, ITEMS, FwdSo
     __device__ Pair<T> identity() const { return {T(0), T(0)}; }
     __device__ Pair<T> combine(const Pair<T> &a, const Pair<T> &b) const {
         return {a.b + b.b + a.c * b.c, a.c + b.c};
+    }
+    static constexpr int kExact = sizeof(T) == 4 ? kExactSum : kExactNone;
+    __device__ void extend(Pair<T> &hi, Pair<T> &lo, const Pair<T> &d) const {
+        const T p = mul_rn(hi.c, d.c);
+        lo.b += fma(hi.c, d.c, -p) + lo.c * d.c;
+        add_carry(hi.b, lo.b, d.b);
+        add_carry(hi.b, lo.b, p);
+        add_carry(hi.c, lo.c, d.c);
     }
 };
 
@@ -200,6 +216,8 @@ template <typename T, int ITEMS> struct VjpAdd {
         load_chunk_sm(sm[0] + lo, c0, n, r.v, T(0));
     }
     static constexpr int kWalk = 0;
+    static constexpr int kExact = sizeof(T) == 4 ? kExactSum : kExactNone;
+    __device__ void extend(T &hi, T &lo, T d) const { add_carry(hi, lo, d); }
     using Scalar = T;
     __device__ T *dst() const { return xbar; }
     __device__ bool accumulating() const { return accumulate != 0; }
@@ -260,6 +278,9 @@ template <typename T, int ITEMS> struct VjpMul {
         fetch_prev_sm(sm[2], lo, c0, n, r.y, T(1));
     }
     static constexpr int kWalk = 1;
+    static constexpr int kExact = sizeof(T) == 4 ? kExactProduct : kExactNone;
+    __device__ static T &coef(State &s) { return s.c; }
+    __device__ static const T &coef(const State &s) { return s.c; }
     using Scalar = T;
     __device__ Elem *dst() const { return xbar; }
     __device__ bool accumulating() const { return accumulate != 0; }
@@ -316,6 +337,13 @@ template <typename T, int ITEMS, bool MAX> struct VjpSel {
         fetch_both_sm(sm[1], lo, c0, n, r.y, T(0));
     }
     static constexpr int kWalk = 2;
+    static constexpr int kExact = sizeof(T) == 4 ? kExactSum : kExactNone;
+    __device__ void extend(State &hi, State &lo, const State &d) const {  // d.c is 0 or 1
+        hi.v *= d.c;
+        lo.v *= d.c;
+        hi.c *= d.c;
+        add_carry(hi.v, lo.v, d.v);
+    }
     using Scalar = T;
     __device__ Elem *dst() const { return xbar; }
     __device__ bool accumulating() const { return accumulate != 0; }
@@ -381,6 +409,9 @@ template <typename T, int ITEMS> struct VjpLin {
         fetch_prev_sm(sm[2], lo, c0, n, r.y, e);
     }
     static constexpr int kWalk = 1;
+    static constexpr int kExact = sizeof(T) == 4 ? kExactProduct : kExactNone;
+    __device__ static T &coef(State &s) { return s.c; }
+    __device__ static const T &coef(const State &s) { return s.c; }
     using Scalar = T;
     __device__ Elem *dst() const { return xbar; }
     __device__ bool accumulating() const { return accumulate != 0; }
@@ -449,6 +480,15 @@ template <typename T, int ITEMS> struct VjpSop {
         fetch_prev_sm(sm[2], lo, c0, n, r.y, z);
     }
     static constexpr int kWalk = 1;
+    static constexpr int kExact = sizeof(T) == 4 ? kExactSum : kExactNone;
+    __device__ void extend(State &hi, State &lo, const State &d) const {
+        const T p = mul_rn(d.sig, hi.vp);
+        lo.vs += fma(d.sig, hi.vp, -p) + d.sig * lo.vp;
+        add_carry(hi.vs, lo.vs, d.vs);
+        add_carry(hi.vs, lo.vs, p);
+        add_carry(hi.vp, lo.vp, d.vp);
+        hi.sig += d.sig;
+    }
     using Scalar = T;
     __device__ Elem *dst() const { return xbar; }
     __device__ bool accumulating() const { return accumulate != 0; }
@@ -810,11 +850,11 @@ static adc_status launch(const Op &o, int64_t n, void *ws, cudaStream_t s) {
 // The streaming engine's shape per operator (n = 1e8 fp32, n = 1e7 fp64; the
 // figures are this shape's against the next best one measured).  One input
 // array: 128-byte rows, 6 stages of 32 KB, fold and store by the same warps
-// (+ 0.138 / lin 0.284 ms forward; split 0.148 / 0.296).  The vjps of two and
+// (+ 0.136 / lin 0.282 ms forward; split 0.148 / 0.296).  The vjps of two and
 // three arrays: 64-byte rows, 4 stages of up to 48 KB; in fp32 the smem left is
 // short of the look-back's latency, and separate fold and store warps make up
-// for part of it (lin vjp 0.617 ms; same warps 0.721); in fp64 the second set of
-// warps only contends for the FP64 pipe (* vjp 0.149 ms; split 0.235).
+// for part of it (lin vjp 0.628 ms; same warps 0.721 before errors were carried); in fp64 the second set of
+// warps only contends for the FP64 pipe (* vjp 0.150 ms; split 0.235).
 template <class Op> struct StreamPick {
     static constexpr bool one = Op::kStreams == 1;
     static constexpr bool f32 = sizeof(typename Op::Scalar) == 4;
@@ -823,7 +863,7 @@ template <class Op> struct StreamPick {
 };
 // From 3 MB per input array on (about one 32 KB tile for every second SM) the
 // streaming engine is the faster one at every size measured: + n = 1e6 0.0139 ->
-// 0.0133 ms, 2e6 0.0214 -> 0.0157, 1e7 0.0352 -> 0.0235, 1e8 0.215 -> 0.138;
+// 0.0133 ms, 2e6 0.0214 -> 0.0157, 1e7 0.0352 -> 0.0235, 1e8 0.215 -> 0.136;
 // below, both are bound by their launches and the per-tile engine has the
 // smaller blocks.  A tuned range length asks for the range engine.
 constexpr int64_t kStreamMinBytes = 3 << 20;

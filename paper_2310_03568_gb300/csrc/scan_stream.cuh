@@ -23,7 +23,7 @@
 // bandwidth, during which its inputs wait in shared memory.  With one input
 // array six 32 KB stages cover it (n = 1e8 fp32 + forward 0.136 ms, 0.87 of the
 // 6.8 TB/s copy rate; the range engine, which reads the input twice, 0.215);
-// with three arrays four 48 KB stages do not (lin vjp 0.612 ms, 0.77; 0.764).
+// with three arrays four 48 KB stages do not (lin vjp 0.628 ms, 0.75; 0.764).
 // Hence: four copies of the aggregates, so that fewer blocks poll the same
 // lines (lin vjp 0.90 -> 0.72 ms before the roles were split); claims at the
 // pace of the folds (claimed in bursts, a block folds neighbouring tiles a
@@ -44,9 +44,12 @@
 //   kWalk 1: item(a, xn)        a = stream 0 at i, xn = stream 1 at i + 1;
 //            out(run, yp)       yp = stream 2 at i - 1
 //   kWalk 2: item(a, y, yn, i, n), out(run, y, yp, i)   a = stream 0, y = stream 1
+//   kExact (0 if absent)        which fp32 roundings are carried along, below
 #pragma once
 
+#include <cfloat>
 #include <string.h>
+#include <type_traits>
 
 #include "common.cuh"
 #include "internal.h"
@@ -149,6 +152,106 @@ __device__ __forceinline__ void copy16(unsigned char *dst, const E *src, int64_t
     *reinterpret_cast<uint4 *>(dst) = t;
 }
 
+// fp32 roundings that are carried along (Op::kExact).
+// kExactProduct: the state's coefficient coef(s) is the product of the elements'
+// coefficients.  The relative error of a product is the sum of the roundings of
+// all its multiplications, in whatever order they are done, so where a linear
+// recurrence grows over tens of thousands of elements, 1e-6 to 6e-6 of the result
+// was rounding.  A tile's fold keeps each multiplication's error (an FMA gives it)
+// beside the coefficient, two FMAs per element, and rounds once per tile: 1e-7 to
+// 5e-7 (lin, n = 1e6 to 1e8), for 2% to 10% of the time (n = 1e8 lin vjp 0.612 ->
+// 0.628 ms, * vjp 0.293 -> 0.321; the range engine 0.764 and 0.41).  Without bringing
+// the coefficient to the nearest after every combine, lin
+// 0.617 ms but errors up to 1.2e-6.
+// kExactSum: the block's running prefix is extended once per round of tiles, at
+// its own magnitude: 160 roundings over n = 1e8.  extend(hi, lo, d) sums up
+// their errors beside it (sumOfProd n = 5e7: 5.7e-7 -> 2.4e-7, as without tiles).
+// A coefficient or prefix that is not finite carries no error: NaN and
+// infinities come out as without it.
+enum { kExactNone = 0, kExactProduct = 1, kExactSum = 2 };
+template <class Op, class = void> struct ExactOf : std::integral_constant<int, kExactNone> {};
+template <class Op> struct ExactOf<Op, std::void_t<decltype(Op::kExact)>> : std::integral_constant<int, Op::kExact> {};
+
+// hi += d, the rounding error added to lo (two-sum; Knuth, TAOCP 2, 4.2.2).
+template <typename T> __device__ __forceinline__ void add_carry(T &hi, T &lo, T d) {
+    const T a = hi, s = a + d, b = s - a;
+    lo += (a - (s - b)) + (d - b);
+    hi = s;
+}
+
+// A product that is rounded before it is used, never contracted into an FMA.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
+// What a tile's fold carries: the state, and its coefficient's error.
+template <class Op, bool PRODUCT = ExactOf<Op>::value == kExactProduct> struct TileFold {
+    using S = typename Op::State;
+    using X = S;
+    const Op &op;
+    __device__ X identity() const { return op.identity(); }
+    __device__ X step(const X &a, const S &x) const { return op.combine(a, x); }  // one more element
+    __device__ X sealed(const X &a) const { return a; }                           // after the last one
+    __device__ X combine(const X &a, const X &b) const { return op.combine(a, b); }
+    __device__ static const S &state(const X &a) { return a; }
+};
+template <class Op> struct TileFold<Op, true> {
+    using S = typename Op::State;
+    struct X {
+        S s;
+        float e;
+    };
+    const Op &op;
+    __device__ X identity() const { return {op.identity(), 0.f}; }
+    __device__ X step(const X &a, const S &x) const {
+        const float ac = Op::coef(a.s), xc = Op::coef(x), c = __fmul_rn(xc, ac);
+        X r{op.combine(a.s, x), fmaf(xc, a.e, fmaf(xc, ac, -c))};
+        Op::coef(r.s) = c;
+        return r;
+    }
+    __device__ X sealed(X r) const {  // the coefficient to the nearest, what is left in e
+        const float c = Op::coef(r.s), t = __fadd_rn(c, r.e);
+        if (r.e != 0.f && fabsf(t) <= FLT_MAX) {
+            Op::coef(r.s) = t;
+            r.e = __fsub_rn(r.e, __fsub_rn(t, c));
+        } else {
+            r.e = 0.f;
+        }
+        return r;
+    }
+    __device__ X combine(const X &a, const X &b) const {
+        X r = step(a, b.s);
+        r.e = fmaf(b.e, Op::coef(a.s), r.e);
+        return sealed(r);
+    }
+    __device__ static const S &state(const X &a) { return a.s; }
+};
+
+// The block's running prefix.
+template <class Op, bool SUM = ExactOf<Op>::value == kExactSum> struct RunningPrefix {
+    using S = typename Op::State;
+    S run;
+    __device__ explicit RunningPrefix(const Op &op) : run(op.identity()) {}
+    __device__ void extend(const Op &op, const S &d) { run = op.combine(run, d); }
+    __device__ S value() const { return run; }
+};
+template <class Op> struct RunningPrefix<Op, true> {
+    using S = typename Op::State;
+    S run, lo;
+    __device__ explicit RunningPrefix(const Op &op) : run(op.identity()) { memset(&lo, 0, sizeof(S)); }
+    __device__ void extend(const Op &op, const S &d) { op.extend(run, lo, d); }
+    __device__ S value() const {
+        S out;
+        const float *h = reinterpret_cast<const float *>(&run), *l = reinterpret_cast<const float *>(&lo);
+        float *o = reinterpret_cast<float *>(&out);
+#pragma unroll
+        for (int k = 0; k < (int)(sizeof(S) / 4); ++k) {
+            const float t = __fadd_rn(h[k], l[k]);
+            o[k] = fabsf(t) <= FLT_MAX ? t : h[k];
+        }
+        return out;
+    }
+};
+
 // Folds the aggregates of tiles [from, to) in order onto *run (a whole warp;
 // uniform result); false, alike in every lane, if a bounded wait ran out.
 // Word k of tile t is aggw[k * stride + t].  Every lane polls its own words
@@ -159,10 +262,11 @@ __device__ __forceinline__ void copy16(unsigned char *dst, const E *src, int64_t
 // part's FP64 pipe: 0.090 -> 0.069 ms for the n = 1e7 * forward).  Handing the
 // tiles over through shared memory to have both was slower for fp32 (0.148 ->
 // 0.160 ms, n = 1e8 +): it lengthens the one chain that everything waits for.
-template <class Op, typename S>
+template <class Op>
 __device__ __forceinline__ bool stream_lookback(const Op &op, const unsigned long long *__restrict__ aggw,
-                                                unsigned stride, unsigned from, unsigned to, S *run,
-                                                long long limit) {
+                                                unsigned stride, unsigned from, unsigned to,
+                                                RunningPrefix<Op> *run, long long limit) {
+    using S = typename Op::State;
     constexpr int K = Tagged<S>::K;
     constexpr int Q = 5;  // 160 tiles: one per SM, so one step as a rule
     constexpr bool kLaneMajor = K > 4 || sizeof(typename Op::Scalar) == 8;
@@ -216,7 +320,12 @@ __device__ __forceinline__ bool stream_lookback(const Op &op, const unsigned lon
             }
         }
 #pragma unroll
-        for (int q = 0; q < (kLaneMajor ? 1 : Q); ++q) *run = op.combine(*run, shfl_idx(v[q], 0));
+        for (int q = 0; q < (kLaneMajor ? 1 : Q); ++q) v[q] = shfl_idx(v[q], 0);
+        if constexpr (!kLaneMajor) {
+#pragma unroll
+            for (int q = 1; q < Q; ++q) v[0] = op.combine(v[0], v[q]);
+        }
+        run->extend(op, v[0]);
     }
     return true;
 }
@@ -232,13 +341,16 @@ k_scan_stream(const Op op, const int64_t n, const int64_t num_tiles, unsigned lo
     using T = typename Op::Scalar;
     using Sh = StreamShape<Op, NWC, RB, STAGES>;
     using Seg = Segment<Sh, RB>;
+    using X = typename TileFold<Op>::X;
+    const TileFold<Op> tf{op};
     constexpr int K = Tagged<S>::K;
     constexpr int RING = 2 * STAGES;  // claimed tiles remembered
     static_assert(AHEAD >= 1 && AHEAD < STAGES && NWC <= 32, "loads in flight, and a stage for the tile being folded");
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(8) unsigned long long s_bar_agg[STAGES], s_bar_pre[STAGES], s_bar_free[STAGES],
         s_bar_claim[RING];
-    __shared__ S s_agg[STAGES][NWC], s_wex[STAGES][NWC], s_pre[STAGES];
+    __shared__ X s_agg[STAGES][NWC];
+    __shared__ S s_wex[STAGES][NWC], s_pre[STAGES];
     __shared__ unsigned s_tile[RING];
     __shared__ volatile int s_abort;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -276,7 +388,7 @@ k_scan_stream(const Op op, const int64_t n, const int64_t num_tiles, unsigned lo
     constexpr int kWorkers = SPLIT ? 2 * NWC : NWC;
     if (warp == kWorkers + 1) {  // -------------------------------------- look-back --
         const unsigned long long *mine = aggw + (size_t)(blockIdx.x % reps) * T_ * K;
-        S run = op.identity();  // the exclusive prefix of tile `from`
+        RunningPrefix<Op> run(op);  // the exclusive prefix of tile `from`
         unsigned from = 0;
         for (unsigned i = 0;; ++i) {
             if (!wait_ring(s_bar_claim, i, RING)) return;
@@ -287,7 +399,7 @@ k_scan_stream(const Op op, const int64_t n, const int64_t num_tiles, unsigned lo
             // once the tile itself is folded, the previous use of its slots is over
             if (!ok || !wait_ring(s_bar_agg, i, STAGES)) return;
             if (lane == 0) {
-                s_pre[i % STAGES] = run;
+                s_pre[i % STAGES] = run.value();
                 mbar_arrive(&s_bar_pre[i % STAGES]);
             }
             from = t;
@@ -310,8 +422,10 @@ k_scan_stream(const Op op, const int64_t n, const int64_t num_tiles, unsigned lo
             if (!wait_ring(s_bar_claim, i, RING)) return;
             const unsigned t = s_tile[i % RING];
             if (t >= T_ || !wait_ring(s_bar_agg, i, STAGES)) return;
-            const S inc = warp_inclusive_scan(op, lane < NWC ? s_agg[i % STAGES][lane] : op.identity());
-            const S total = shfl_idx(inc, NWC - 1);
+            X incx = lane < NWC ? s_agg[i % STAGES][lane] : tf.identity();
+#pragma unroll
+            for (int o = 1; o < NWC; o <<= 1) shfl_combine(tf, incx, o, false, lane >= o);
+            const S inc = tf.state(incx), total = shfl_idx(inc, NWC - 1);
             if (lane < reps && (long long)t != ctl.stall_tile) {
                 const unsigned *w = reinterpret_cast<const unsigned *>(&total);
 #pragma unroll
@@ -395,7 +509,7 @@ k_scan_stream(const Op op, const int64_t n, const int64_t num_tiles, unsigned lo
         cp_async_wait<AHEAD - 1>();
         __syncwarp();
         const int64_t e0 = first_byte(t) / (int64_t)sizeof(E) + (int64_t)row * Sh::EPR;
-        S a = op.identity();
+        X a = tf.identity();
         const Seg s0 = segment(i, 0);
         if constexpr (Op::kWalk == 0) {
 #pragma unroll
@@ -403,7 +517,7 @@ k_scan_stream(const Op op, const int64_t n, const int64_t num_tiles, unsigned lo
                 E v[Sh::NPU];
                 s0.load(row, REVERSE ? Sh::UR - 1 - uu : uu, v);
 #pragma unroll
-                for (int kk = 0; kk < Sh::NPU; ++kk) a = op.combine(a, op.item(v[REVERSE ? Sh::NPU - 1 - kk : kk]));
+                for (int kk = 0; kk < Sh::NPU; ++kk) a = tf.step(a, op.item(v[REVERSE ? Sh::NPU - 1 - kk : kk]));
             }
         } else {
             static_assert(Op::kWalk == 0 || REVERSE, "the vjp walks run in descending order");
@@ -417,14 +531,14 @@ k_scan_stream(const Op op, const int64_t n, const int64_t num_tiles, unsigned lo
 #pragma unroll
                 for (int k = Sh::NPU - 1; k >= 0; --k) {
                     const E nx = k + 1 < Sh::NPU ? x[k + 1 < Sh::NPU ? k + 1 : 0] : xn;
-                    if constexpr (Op::kWalk == 1) a = op.combine(a, op.item(v[k], nx));
-                    else a = op.combine(a, op.item(v[k], x[k], nx, e0 + u * Sh::NPU + k, n));
+                    if constexpr (Op::kWalk == 1) a = tf.step(a, op.item(v[k], nx));
+                    else a = tf.step(a, op.item(v[k], x[k], nx, e0 + u * Sh::NPU + k, n));
                 }
                 xn = x[0];
             }
         }
-        const S inc = warp_inclusive_scan(op, a);
-        S ex = shfl_up(inc, 1);
+        const X inc = warp_inclusive_scan(tf, tf.sealed(a));
+        S ex = shfl_up(tf.state(inc), 1);
         if (lane == 0) ex = op.identity();
         if (lane == kWarp - 1) s_agg[i % STAGES][w] = inc;
         s_ex[(i % STAGES) * NWC * 32] = ex;
