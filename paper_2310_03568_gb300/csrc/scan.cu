@@ -853,8 +853,9 @@ static adc_status launch(const Op &o, int64_t n, void *ws, cudaStream_t s) {
 // (+ 0.136 / lin 0.282 ms forward; split 0.148 / 0.296).  The vjps of two and
 // three arrays: 64-byte rows, 4 stages of up to 48 KB; in fp32 the smem left is
 // short of the look-back's latency, and separate fold and store warps make up
-// for part of it (lin vjp 0.628 ms; same warps 0.721 before errors were carried); in fp64 the second set of
-// warps only contends for the FP64 pipe (* vjp 0.150 ms; split 0.235).
+// for part of it (lin vjp 0.612 ms, same warps 0.721, both before the products'
+// errors were carried); in fp64 the second set of warps only contends for the
+// FP64 pipe (* vjp 0.150 ms; split 0.235).
 template <class Op> struct StreamPick {
     static constexpr bool one = Op::kStreams == 1;
     static constexpr bool f32 = sizeof(typename Op::Scalar) == 4;

@@ -23,7 +23,7 @@
 // bandwidth, during which its inputs wait in shared memory.  With one input
 // array six 32 KB stages cover it (n = 1e8 fp32 + forward 0.136 ms, 0.87 of the
 // 6.8 TB/s copy rate; the range engine, which reads the input twice, 0.215);
-// with three arrays four 48 KB stages do not (lin vjp 0.628 ms, 0.75; 0.764).
+// with three arrays four 48 KB stages do not (lin vjp 0.633 ms, 0.74; 0.764).
 // Hence: four copies of the aggregates, so that fewer blocks poll the same
 // lines (lin vjp 0.90 -> 0.72 ms before the roles were split); claims at the
 // pace of the folds (claimed in bursts, a block folds neighbouring tiles a
@@ -159,10 +159,10 @@ __device__ __forceinline__ void copy16(unsigned char *dst, const E *src, int64_t
 // recurrence grows over tens of thousands of elements, 1e-6 to 6e-6 of the result
 // was rounding.  A tile's fold keeps each multiplication's error (an FMA gives it)
 // beside the coefficient, two FMAs per element, and rounds once per tile: 1e-7 to
-// 5e-7 (lin, n = 1e6 to 1e8), for 2% to 10% of the time (n = 1e8 lin vjp 0.612 ->
-// 0.628 ms, * vjp 0.293 -> 0.321; the range engine 0.764 and 0.41).  Without bringing
-// the coefficient to the nearest after every combine, lin
-// 0.617 ms but errors up to 1.2e-6.
+// 8e-7 (lin, n = 1e6 to 1e8), for 3% to 10% of the vjps' time (n = 1e8 lin 0.612 ->
+// 0.633 ms, * 0.293 -> 0.321; the range engine 0.764 and 0.41).  Without bringing
+// the coefficient to the nearest after every combine, lin took 0.619 ms, but with
+// errors up to 1.2e-6.
 // kExactSum: the block's running prefix is extended once per round of tiles, at
 // its own magnitude: 160 roundings over n = 1e8.  extend(hi, lo, d) sums up
 // their errors beside it (sumOfProd n = 5e7: 5.7e-7 -> 2.4e-7, as without tiles).

@@ -938,8 +938,8 @@ k_vscan_wfold(const Op op, const int64_t n, const int64_t d, const int64_t U, ty
 // this kernel is a chain of latencies: at d = 16 and about 9700 units, reading
 // every unit's state at a stride of d states took 28 us.  With up to one state
 // per thread the units' own states are as quick to read, and the fold's barrier
-// and its units in order are saved (n = 22,514, d = 12, forward + vjp: 0.045 ->
-// 0.040 ms).
+// and its units in order are saved (n = 22,514, d = 12, forward + vjp: 0.0450 ->
+// 0.0427 ms).
 constexpr int kVPrefixThreads = 1024;
 template <class Op>
 __global__ void __launch_bounds__(kVPrefixThreads)
