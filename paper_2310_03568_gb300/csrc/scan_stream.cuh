@@ -545,8 +545,16 @@ k_scan_stream(const Op op, const int64_t n, const int64_t num_tiles, unsigned lo
         __syncwarp();
         if (lane == kWarp - 1) mbar_arrive(&s_bar_agg[i % STAGES]);
     };
+    // fp32 sums: a row's elements are summed from zero and the row's prefix is
+    // added to each partial sum.  Added to the prefix one by one, each of a row's 32
+    // elements rounds at the prefix's magnitude: 1.1e-7 of the results for values
+    // in (-1, 1) at n = 2^24 (16-element rows 8e-8), from zero 3.7e-8.  The pass is
+    // bound by memory: n = 1e8 forward + vjp 0.267 ms before, 0.268 with it.
+    constexpr bool kFromBase = Op::kWalk == 0 && ExactOf<Op>::value == kExactSum && std::is_same<S, float>::value;
     const auto store = [&](unsigned j) {
-        S run = op.combine(op.combine(s_pre[j % STAGES], s_wex[j % STAGES][w]), s_ex[(j % STAGES) * NWC * 32]);
+        const S pre = s_pre[j % STAGES], wex = s_wex[j % STAGES][w], ex = s_ex[(j % STAGES) * NWC * 32];
+        S run = kFromBase ? op.combine(pre, op.combine(wex, ex)) : op.combine(op.combine(pre, wex), ex);
+        S loc = op.identity();
         const int64_t b0 = first_byte(s_tile[j % RING]);
         const int64_t e0 = b0 / (int64_t)sizeof(E) + (int64_t)row * Sh::EPR;
         const Seg s0 = segment(j, 0);
@@ -559,8 +567,13 @@ k_scan_stream(const Op op, const int64_t n, const int64_t num_tiles, unsigned lo
 #pragma unroll
                 for (int kk = 0; kk < Sh::NPU; ++kk) {
                     const int k = REVERSE ? Sh::NPU - 1 - kk : kk;
-                    run = op.combine(run, op.item(v[k]));
-                    v[k] = op.out(run, e0 + u * Sh::NPU + k);
+                    if constexpr (kFromBase) {
+                        loc = op.combine(loc, op.item(v[k]));
+                        v[k] = op.out(op.combine(run, loc), e0 + u * Sh::NPU + k);
+                    } else {
+                        run = op.combine(run, op.item(v[k]));
+                        v[k] = op.out(run, e0 + u * Sh::NPU + k);
+                    }
                 }
                 s0.store(row, u, v);
             }

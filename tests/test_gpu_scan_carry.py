@@ -63,3 +63,21 @@ def test_infinities_stay_infinite(op):
     y = host(adcomb.scan_fwd(op, dev(x if w == 2 else x[:, 0]))).reshape(N, w)
     # (for *, 0.5^i underflows to 0 long before, and 0 * inf is NaN)
     assert np.isfinite(y[:at]).all() and not np.isfinite(y[at:]).any()
+
+
+@pytest.mark.parametrize("direction", ["fwd", "vjp"])
+def test_small_elements_after_a_large_prefix(direction):
+    """2^25 (whose unit in the last place is 4), zeros to the end of the 8192-element
+    tile, then halves: every row's, tile's and running sum is a multiple of 16 below
+    2^26, so exact, and a result rounds once, by at most 2."""
+    n = 128 * 8192
+    x = np.full(n, 0.5, np.float32)
+    x[:8192] = 0
+    x[0] = 2.0**25
+    ref = np.cumsum(x.astype(np.float64))
+    if direction == "fwd":
+        got = host(adcomb.scan_fwd("add", dev(x)))
+    else:
+        r = dev(x[::-1].copy())
+        got = host(adcomb.scan_vjp("add", r, r, r))[::-1]
+    assert np.max(np.abs(got - ref)) <= 2
