@@ -405,7 +405,9 @@ void adc_set_spin_limit(int64_t iterations);
 /*
  * Fault-injection hook for tests: the scan tile with this claim index
  * publishes nothing, so every tile that looks back across it must give up
- * after the spin limit and report ADC_ERR_TIMEOUT.  -1 (the default) disables.
+ * after the spin limit and report ADC_ERR_TIMEOUT.  In the partitioned
+ * reduce_by_index (fp32) it is a chunk of 8192 elements whose copy into shared
+ * memory never comes.  -1 (the default) disables.
  */
 void adc_debug_set_stall_tile(int64_t tile);
 

@@ -15,8 +15,6 @@ int g_scan_engine = 0;
 int g_scan_range_tiles = 0;
 int g_scan_prefetch = 0;
 
-long long spin_limit() { return g_spin_limit; }
-
 DevCtl make_ctl(void *ws, int slot) {
     DevCtl c;
     c.err = static_cast<unsigned *>(ws);

@@ -443,7 +443,7 @@ __global__ void __launch_bounds__(kScatThreads, 2)
 k_part_scatter_tma(const int32_t *__restrict__ keys, const float *__restrict__ vals, const int64_t n, const int64_t m,
                    const BucketDiv bdiv, const int B, const int64_t nchunks, int32_t *__restrict__ cursor,
                    uint16_t *__restrict__ obin, typename PartTraits<float, MODE>::V *__restrict__ oval,
-                   unsigned *__restrict__ err, const long long spin_limit) {
+                   const DevCtl ctl) {
     using Tr = PartTraits<float, MODE>;
     constexpr int NW = kScatThreads / kWarp;
     constexpr int PER = kPartMaxBuckets / kScatThreads;  // buckets per thread in the local scan
@@ -460,6 +460,7 @@ k_part_scatter_tma(const int32_t *__restrict__ keys, const float *__restrict__ v
     const int64_t G = gridDim.x;
     const auto whole = [&](int64_t c) { return (c + 1) * (int64_t)kPartChunk <= n; };
     const auto issue = [&](int64_t c) {  // thread 0
+        if (c == ctl.stall_tile) return;  // fault injection: a copy that never comes
         fence_proxy_async_smem();
         mbar_expect_tx(&s_bar, 2u * kChunkBytes);
         bulk_g2s(sk, keys + c * kPartChunk, kChunkBytes, &s_bar);
@@ -477,15 +478,15 @@ k_part_scatter_tma(const int32_t *__restrict__ keys, const float *__restrict__ v
         const int64_t e0 = c * kPartChunk;
         const int len = (int)((n - e0) < kPartChunk ? (n - e0) : kPartChunk);
         if (whole(c)) {
-            const bool ok = mbar_wait_bounded(&s_bar, used & 1u, spin_limit);
-            ++used;
-            if (!__syncthreads_and(ok)) {  // report, give the copy a second bounded wait, leave
+            const bool ok = mbar_wait_bounded(&s_bar, used & 1u, ctl.spin_limit);
+            if (!__syncthreads_and(ok)) {  // report, let the copy land, leave: the table pass touches nothing
                 if (tid == 0) {
-                    set_error(err, kErrTimeout);
-                    mbar_wait_bounded(&s_bar, (used - 1u) & 1u, spin_limit);
+                    set_error(ctl.err, kErrTimeout);
+                    if (c != ctl.stall_tile) mbar_drain(&s_bar, used & 1u);
                 }
                 return;
             }
+            ++used;
         } else {
             for (int i = tid; i < len; i += kScatThreads) {
                 sk[i] = keys[e0 + i];
@@ -572,7 +573,10 @@ k_part_scatter_tma(const int32_t *__restrict__ keys, const float *__restrict__ v
 }
 
 // 3. One block per bucket: the bucket's W bins in shared memory, its run of
-// (bin, payload) streamed in, the bins written out.
+// (bin, payload) streamed in, the bins written out.  A scatter block that gave
+// up on its copy left its share of the runs unwritten, and what lies there is
+// neither a bin nor an element: with a timeout recorded, no element is touched
+// and every bin comes out empty.
 template <typename T, int MODE>
 __global__ void __launch_bounds__(kPartTableThreads)
 k_part_table(const uint16_t *__restrict__ obin, const typename PartTraits<T, MODE>::V *__restrict__ oval,
@@ -586,7 +590,7 @@ k_part_table(const uint16_t *__restrict__ obin, const typename PartTraits<T, MOD
     for (int t = threadIdx.x; t < w; t += kPartTableThreads) Tr::init(smem_raw, (int)W, t);
     __syncthreads();
     const int64_t start = bucket[blockIdx.x];
-    const int64_t end = bucket[blockIdx.x + 1];
+    const int64_t end = (__ldcg(err) & kErrTimeout) ? start : bucket[blockIdx.x + 1];
     constexpr int U = 8;
     for (int64_t g0 = start; g0 < end; g0 += (int64_t)U * kPartTableThreads) {
         int32_t u[U];
@@ -710,7 +714,7 @@ static adc_status part_run(int64_t n, int64_t m, const int32_t *keys, const T *v
         if (!smem_attr(k_part_scatter_tma<MODE>, sm_tma)) return ADC_ERR_CUDA;
         const int64_t two = (int64_t)num_sms() * 2;
         k_part_scatter_tma<MODE><<<(unsigned)(nc < two ? nc : two), kScatThreads, sm_tma, s>>>(
-            keys, vals, n, m, bdiv, P.B, nc, cursor, obin, oval, err, spin_limit());
+            keys, vals, n, m, bdiv, P.B, nc, cursor, obin, oval, make_ctl(ws, kPartSlot));
     } else {
         const size_t sm_scatter = (size_t)kPartChunk * (sizeof(V) + 4) + (size_t)P.B * 8;
         if (!smem_attr(k_part_scatter<T, MODE>, sm_scatter)) return ADC_ERR_CUDA;

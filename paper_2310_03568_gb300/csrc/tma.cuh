@@ -45,6 +45,13 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned long long *bar, uint3
     return true;
 }
 
+// The wait of a block that gives up for its own copy in flight: a copy that
+// lands after the block has left would write into another block's shared
+// memory.  Its limit is its own, since the one that ran out may be short.
+__device__ __forceinline__ void mbar_drain(unsigned long long *bar, uint32_t parity) {
+    mbar_wait_bounded(bar, parity, 1ll << 22);
+}
+
 // Orders this thread's earlier generic-proxy shared-memory accesses before
 // later async-proxy (bulk copy) accesses: issued before refilling a buffer
 // that threads have just read.
