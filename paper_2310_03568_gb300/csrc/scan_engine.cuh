@@ -36,6 +36,7 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "tma.cuh"
 
 namespace adc {
 
@@ -66,8 +67,8 @@ template <class Op> constexpr auto op_dyn_smem(int) -> decltype(Op::kDynSmem, si
 // the tile, op.fetch() has thread 0 issue the copies, and every thread then
 // waits through op.staged_wait(limit), bounded, before build().  A wait that
 // runs out marks the tile ERROR and records kErrTimeout, as a look-back that
-// runs out does; thread 0 then gives the copies a second bounded wait before
-// the block leaves.
+// runs out does; thread 0 then waits for the copies to land (kDrainLimit)
+// before the block leaves.
 template <class Op> constexpr bool bulk_staged(long) { return false; }
 template <class Op> constexpr auto bulk_staged(int) -> decltype(Op::kBulkStaged, bool()) { return Op::kBulkStaged; }
 // Such an Op may also finish its tile after store() (kFinish: e.g. stage a
@@ -290,7 +291,7 @@ k_scan(const Op op, const int64_t n, const int64_t num_tiles, unsigned long long
                 if (tid == 0) {
                     publish_tag(incw + t * SO, K, kFlagError, WS);
                     set_error(ctl.err, kErrTimeout);
-                    op.staged_wait(ctl.spin_limit);
+                    op.staged_wait(kDrainLimit);  // no copy in flight when the block leaves
                 }
                 return;
             }

@@ -24,7 +24,7 @@
 // Elements outside the array are never read from it: the vjp's x_n (after the
 // last element) and y_{-1} (before the first) are the identity, written into
 // the stage by thread 0.  Every wait on a copy is bounded (the engine's spin
-// limit); a block whose wait runs out gives the copy a second bounded wait
+// limit); a block whose wait runs out lets the copy land (a limit of its own)
 // before it leaves, and the call reports a timeout.
 #pragma once
 
@@ -315,7 +315,7 @@ template <typename T, int Q, int TH, int SEG> struct StagedVjpMMQ {
             if (e0 == 0) put_eye<T, Q>(reinterpret_cast<T *>(base + kOffX + G::H - G::B));
         }
         if (!__syncthreads_and(mbar_wait_bounded(bar(1), 0u, limit))) {
-            if (threadIdx.x == 0) mbar_wait_bounded(bar(1), 0u, limit);  // a second chance for the copy to land
+            if (threadIdx.x == 0) mbar_drain(bar(1), 0u);
             return false;
         }
         // Mbar_i = P_{i-1}^T lambda_i, one element per thread, in place of lambda_i

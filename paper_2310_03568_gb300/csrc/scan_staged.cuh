@@ -317,13 +317,13 @@ k_scan_staged(const Op op, const int64_t n, const int64_t num_tiles, const int r
         }
     }
     if (abort && tid == 0) {
-        // leave no bulk copy in flight into this block's shared memory: give the
-        // current range's and the prefetched range's copies a bounded chance to land
+        // leave no bulk copy in flight into this block's shared memory: the current
+        // range's and the prefetched range's copies land first
         const int buf = (int)(i & 1);
         for (int g = 0; g < kStageGroups; ++g) {
-            mbar_wait_bounded(&s_bar[buf][g], (uint32_t)((i >> 1) & 1), ctl.spin_limit);
+            mbar_drain(&s_bar[buf][g], (uint32_t)((i >> 1) & 1));
             if ((long long)(blockIdx.x + (i + 1) * G) < NR)
-                mbar_wait_bounded(&s_bar[buf ^ 1][g], (uint32_t)(((i + 1) >> 1) & 1), ctl.spin_limit);
+                mbar_drain(&s_bar[buf ^ 1][g], (uint32_t)(((i + 1) >> 1) & 1));
         }
     }
 }

@@ -118,7 +118,7 @@ k_scan_tma(const Op op, const int64_t n, const int64_t num_tiles, unsigned long 
         if (tid == 0) {
             publish_tag(incw + t * SO, K, kFlagError, WS);
             set_error(ctl.err, kErrTimeout);
-            mbar_wait_bounded(&s_bar, 0u, ctl.spin_limit);  // a second chance for the copy to land
+            mbar_drain(&s_bar, 0u);
         }
         return;
     }

@@ -48,8 +48,9 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned long long *bar, uint3
 // The wait of a block that gives up for its own copy in flight: a copy that
 // lands after the block has left would write into another block's shared
 // memory.  Its limit is its own, since the one that ran out may be short.
+constexpr long long kDrainLimit = 1ll << 22;
 __device__ __forceinline__ void mbar_drain(unsigned long long *bar, uint32_t parity) {
-    mbar_wait_bounded(bar, parity, 1ll << 22);
+    mbar_wait_bounded(bar, parity, kDrainLimit);
 }
 
 // Orders this thread's earlier generic-proxy shared-memory accesses before
