@@ -96,15 +96,29 @@ template <int ITEMS> struct ExclAddI32 {
 constexpr int kCountItems = 16;
 
 // ---------------------------------------------------------------- scatter --
+// After a timeout in the count matrix's scan the offsets are whatever lay in
+// the workspace.  Nothing is moved by them then: every element stays where it
+// is, with no bin (key m), so that the residuals hold only keys and places
+// that the scans and the vjp may follow.
 template <typename V>
 __global__ void __launch_bounds__(kSortThreads)
 k_sort_scatter(const int32_t *__restrict__ keys, const int32_t *__restrict__ perm_in, const int64_t n, const int64_t m,
                const int first, const SortPass P, const int64_t T, const int32_t *__restrict__ offsets,
                int32_t *__restrict__ keys_out, int32_t *__restrict__ perm_out, const V *__restrict__ vals,
-               V *__restrict__ vals_out) {
+               V *__restrict__ vals_out, const unsigned *__restrict__ err) {
     extern __shared__ int32_t s_w[];  // [8 warps][buckets]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int NW = kSortThreads / kWarp;
+    if (__ldcg(err) != 0u) {
+        for (int r = 0; r < kSortRounds; ++r) {
+            const int64_t i = (int64_t)blockIdx.x * kSortTile + (int64_t)r * kSortThreads + threadIdx.x;
+            if (i >= n) break;
+            keys_out[i] = (int32_t)m;
+            perm_out[i] = (int32_t)i;
+            if (vals_out) vals_out[i] = vals[i];
+        }
+        return;
+    }
     for (int j = threadIdx.x; j < NW * P.buckets; j += kSortThreads) s_w[j] = 0;
     __syncthreads();
     int32_t *wc = s_w + warp * P.buckets;
@@ -439,7 +453,7 @@ static adc_status sort_by_key(int64_t n, int64_t m, const int32_t *keys, const P
             return ADC_ERR_CUDA;
         k_sort_scatter<Pair<T>><<<(unsigned)NT, kSortThreads, ss, s>>>(
             kin, pin, n, m, p == 0, P[p], NT, offs, kb[dst], pb[dst], vals,
-            last ? static_cast<Pair<T> *>(out.svals) : nullptr);
+            last ? static_cast<Pair<T> *>(out.svals) : nullptr, static_cast<const unsigned *>(ws));
         if ((st = check_launch()) != ADC_OK) return st;
         kin = kb[dst];
         pin = pb[dst];

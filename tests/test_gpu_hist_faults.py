@@ -70,3 +70,31 @@ def test_partitioned_chunk_that_never_comes(op, stall):
     ref = oracle.hist_fwd(op, m, keys, v)
     # about 10 positive values a bin, at most some 40: 40 roundings of 2^-24
     np.testing.assert_allclose(host(hist), ref[0] if isinstance(ref, tuple) else ref, rtol=2.5e-6, atol=0)
+
+
+@pytest.mark.parametrize("m,forced", [(5000, -1), (100, 2)], ids=["two-pass", "one-pass"])
+def test_sorted_path_without_offsets(m, forced):
+    """linFnComp through the radix sort: the scan of the counts times out, so no element has a destination."""
+    g = np.random.default_rng(13)
+    n = 300_000
+    keys = g.integers(0, m, n).astype(np.int32)
+    v = np.stack([g.standard_normal(n), g.uniform(0.95, 1.05, n)], 1).astype(np.float32)
+    hb = g.standard_normal((m, 2)).astype(np.float32)
+    kd, vd, hbd = dev(keys), dev(v), dev(hb)
+    try:
+        adcomb.debug_force_hist_strategy(forced)
+        ws = ones_workspace("hist", "lin", n, m)
+        hist = torch.full((m, 2), 7.0, device="cuda")
+        saved = torch.full((adcomb.saved_bytes("hist", "lin", torch.float32, n, m),), 255, dtype=torch.uint8,
+                           device="cuda")
+        stalled(lambda: adcomb.hist_fwd("lin", m, kd, vd, None, hist, saved, ws=ws), ws, 0, 2000)  # the counts are two tiles or more
+        assert (host(hist) == np.array([0.0, 1.0], np.float32)).all()
+        # the residuals may be followed: no element has a bin
+        vb, _ = adcomb.hist_vjp("lin", m, kd, vd, None, hist, saved, hbd, ws=ws)
+        assert adcomb.check_device_error(ws) == 0
+        assert (host(vb) == 0).all()
+        adcomb.hist_fwd("lin", m, kd, vd, None, hist, saved, ws=ws)
+        assert adcomb.check_device_error(ws) == 0
+        np.testing.assert_allclose(host(hist), oracle.hist_fwd("lin", m, keys, v).reshape(m, 2), rtol=1e-3, atol=1e-2)
+    finally:
+        adcomb.debug_force_hist_strategy(-1)
