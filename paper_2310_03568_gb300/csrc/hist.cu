@@ -1842,10 +1842,15 @@ static adc_status hist_vjp_t(adc_op op, int64_t n, int64_t m, const int32_t *key
     const unsigned gn = grid_for(n / 4 + 1, 8);
     const unsigned gn8 = grid_for(n / 8 + 1, 8);  // the * vjp: 8 elements per step
     switch (op) {
-    case ADC_OP_ADD:
-        k_hist_add_vjp<T><<<h0b && gm > gn ? gm : gn, 256, 0, s>>>(keys, hb, vb, h0b, n, m, acc,
-                                                                   static_cast<unsigned *>(ws));
+    case ADC_OP_ADD: {
+        unsigned *header = static_cast<unsigned *>(ws);
+        // histbar += histbar, in place: not while the values' adjoints are gathered from it
+        const bool apart = acc && h0b == hb;
+        k_hist_add_vjp<T><<<h0b && gm > gn ? gm : gn, 256, 0, s>>>(keys, hb, vb, apart ? nullptr : h0b, n, m, acc,
+                                                                   header);
+        if (apart) k_hist_add_vjp<T><<<gm, 256, 0, s>>>(keys, hb, vb, h0b, 0, m, acc, header);
         return check_launch();
+    }
     case ADC_OP_MIN:
     case ADC_OP_MAX: {
         const int32_t *is = static_cast<const int32_t *>(saved);
