@@ -1291,15 +1291,17 @@ __global__ void k_hist_mul_vjp(const int32_t *__restrict__ keys, const T *__rest
     }
 }
 
-// The same with the coefficient table of a bin count beyond L1 but within a
-// block in shared memory (one 1024-thread block per SM; the rare zeros read
-// the second table from L2): a gather that missed L1 cost an L2 round trip per
-// element.
-template <typename T>
+// The same (fp32) with the coefficient table in shared memory: one 1024-thread
+// block per SM; the rare zeros read the second table from L2.  A gather that
+// misses L1 costs an L2 round trip per element, but loading the table into
+// every SM costs microseconds, and one block per SM keeps fewer loads in
+// flight: see the rule at the launch.  (fp64 is bound by its divisions: n = 2e7,
+// m = 8,400 to 25,600 took 0.424 ms this way, 0.416 without.)
 __global__ void __launch_bounds__(1024, 1)
-k_hist_mul_vjp_smem(const int32_t *__restrict__ keys, const T *__restrict__ vals, const T *__restrict__ anz,
-                    const T *__restrict__ az, T *__restrict__ vb, const int64_t n, const int64_t m,
+k_hist_mul_vjp_smem(const int32_t *__restrict__ keys, const float *__restrict__ vals, const float *__restrict__ anz,
+                    const float *__restrict__ az, float *__restrict__ vb, const int64_t n, const int64_t m,
                     const int accumulate) {
+    using T = float;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *tab = reinterpret_cast<T *>(smem_raw);
     for (int64_t j = threadIdx.x; j < m; j += blockDim.x) tab[j] = anz[j];
@@ -1310,7 +1312,7 @@ k_hist_mul_vjp_smem(const int32_t *__restrict__ keys, const T *__restrict__ vals
         if (!in_range(k, m)) return T(0);
         return v != T(0) ? div_or_zero(tab[k], v) : __ldg(az + k);
     };
-    constexpr int U = sizeof(T) == 4 ? 4 : 2;  // 4-element groups per thread and step: all their loads issued first
+    constexpr int U = 4;  // 4-element groups per thread and step: all their loads issued first
     const int64_t nv = n / 4;
     for (int64_t v0 = g; v0 < nv; v0 += U * stride) {
         int4 k[U];
@@ -1885,15 +1887,21 @@ static adc_status hist_vjp_t(adc_op op, int64_t n, int64_t m, const int32_t *key
         T *az = reinterpret_cast<T *>(static_cast<char *>(ws) + kWsHeader + align_up((size_t)m * sizeof(T), 256));
         if (n > 0) {
             k_mul_vjp_prep<T><<<gm, 256, 0, s>>>(n0, p, h0, hb, anz, az, m);
-            // a table that misses L1 but fits a block, and enough elements to pay for
-            // loading it into every SM
-            const size_t tab = (size_t)m * sizeof(T);
-            if (tab > 64 * 1024 && tab <= kBlockBudget && n >= 64 * m) {
-                if (!set_smem(k_hist_mul_vjp_smem<T>, tab)) return ADC_ERR_CUDA;
-                k_hist_mul_vjp_smem<T><<<num_sms(), 1024, tab, s>>>(keys, vals, anz, az, vb, n, m, acc);
-            } else {
-                k_hist_mul_vjp<T><<<gn8, 256, 0, s>>>(keys, vals, anz, az, vb, n, m, acc);
+            // a table that misses L1 often enough (96 KB: at 80 KB 4% to 11% slower up
+            // to n = 512 m, at 100 KB 1% to 6% faster) but fits a block, and elements
+            // enough to pay for loading it into every SM (vjp at m = 50,000: n = 64 m
+            // 0.0165 -> 0.0185 ms, 256 m 0.0467 -> 0.0451, 1024 m 0.143 -> 0.132; at
+            // m = 32,768: 64 m 0.0130 -> 0.0143, 256 m 0.0287 on both, 1024 m 0.085 -> 0.079)
+            bool in_smem = false;
+            if constexpr (sizeof(T) == 4) {
+                const size_t tab = (size_t)m * sizeof(T);
+                in_smem = tab > 96 * 1024 && tab <= kBlockBudget && n >= 256 * m;
+                if (in_smem) {
+                    if (!set_smem(k_hist_mul_vjp_smem, tab)) return ADC_ERR_CUDA;
+                    k_hist_mul_vjp_smem<<<num_sms(), 1024, tab, s>>>(keys, vals, anz, az, vb, n, m, acc);
+                }
             }
+            if (!in_smem) k_hist_mul_vjp<T><<<gn8, 256, 0, s>>>(keys, vals, anz, az, vb, n, m, acc);
         }
         if (h0b) k_h0bar_mul<T><<<gm, 256, 0, s>>>(n0, p, hb, h0b, m, acc);
         return check_launch();
