@@ -28,6 +28,7 @@ constexpr int kRedThreads = 256;
 // ------------------------------------------------------------- operators --
 template <typename T> struct RAdd {
     using State = T;
+    using Scalar = T;
     __device__ State identity() const { return T(0); }
     __device__ State combine(State a, State b) const { return a + b; }
     __device__ State lift(T x, int64_t) const { return x; }
@@ -37,6 +38,7 @@ template <typename T> struct MinMaxS { T v; int32_t i; int32_t pad; };
 
 template <typename T, bool MAX> struct RSel {
     using State = MinMaxS<T>;
+    using Scalar = T;
     int32_t n;
     __device__ State identity() const { return {MAX ? -Num<T>::inf() : Num<T>::inf(), n, 0}; }
     // Fig. 5's min^L: better value wins, equal values -> smaller index.
@@ -55,6 +57,7 @@ template <typename T> struct MulS { T p; int32_t z; int32_t pad; };
 // Fig. 3's lifted primal: (count of zeros, product of non-zeros) under (+, *).
 template <typename T> struct RMul {
     using State = MulS<T>;
+    using Scalar = T;
     __device__ State identity() const { return {T(1), 0, 0}; }
     __device__ State combine(const State &a, const State &b) const { return {a.p * b.p, a.z + b.z, 0}; }
     __device__ State lift(T x, int64_t) const { return x == T(0) ? State{T(1), 1, 0} : State{x, 0, 0}; }
@@ -64,6 +67,7 @@ template <typename T> struct RMul {
 // (p1,s1) . (p2,s2) = (p1 + p2 + s1*s2, s1 + s2); associative and commutative.
 template <typename T> struct RSop {
     using State = Pair<T>;
+    using Scalar = T;
     __device__ State identity() const { return {T(0), T(0)}; }
     __device__ State combine(const State &a, const State &b) const { return {a.b + b.b + a.c * b.c, a.c + b.c}; }
     __device__ State lift(const Pair<T> &x, int64_t) const { return x; }
@@ -92,14 +96,21 @@ template <typename T, int Q> struct GMMQ {
 // commutative, so a thread may take any of the tile's elements: it takes
 // 16-byte words t, t + kRedThreads, ..., so that a warp's load covers 512
 // contiguous bytes.  The lifted operators get each element's own index.
-// Bound by bytes in flight: kRedBlocksPerSM blocks of 256 threads with 64
-// bytes each per thread; whole tiles take no bounds checks.  The last block to
+// fp32 is bound by bytes in flight: six blocks of 256 threads per SM with 64
+// bytes each per thread.  fp64 is bound by its pipe, which every block's scan of
+// its threads' states uses too: five blocks for +, four for the larger states
+// (with six, five and four: + n = 5e7 0.124, 0.117 and 0.119 ms; sumOfProd n =
+// 3e6 0.049, 0.043 and 0.041; * n = 2e6 0.0246, 0.0227 and 0.0227, though n = 5e7
+// 0.214, 0.223 and 0.219).  Whole tiles take no bounds checks.  The last block to
 // finish combines the partials in block order and writes y and the residuals
 // (`fin`), so there is no launch after this one.
-constexpr int kRedBlocksPerSM = 6;
+constexpr int kRedBlocksPerSM = 6;  // the most of any
+template <class Op> constexpr int red_blocks() {
+    return sizeof(typename Op::Scalar) == 4 ? kRedBlocksPerSM : sizeof(typename Op::State) == 8 ? 5 : 4;
+}
 
-template <class Op, class Fin, typename T, int ITEMS>
-__global__ void __launch_bounds__(kRedThreads, kRedBlocksPerSM)
+template <class Op, class Fin, typename T, int ITEMS, int BLOCKS>
+__global__ void __launch_bounds__(kRedThreads, BLOCKS)
 k_reduce_simple(const Op op, const Fin fin, const T *__restrict__ x, const int64_t n, const int64_t tiles_per_block,
                 typename Op::State *__restrict__ part, unsigned *__restrict__ ticket) {
     using S = typename Op::State;
@@ -444,8 +455,8 @@ static bool is_general(adc_op op) {
     return op == ADC_OP_LIN || op == ADC_OP_MM2 || op == ADC_OP_MM3 || op == ADC_OP_MM5;
 }
 
-static int64_t simple_grid(int64_t tiles) {
-    int64_t g = (int64_t)num_sms() * kRedBlocksPerSM;
+static int64_t simple_grid(int64_t tiles, int blocks_per_sm) {
+    int64_t g = (int64_t)num_sms() * blocks_per_sm;
     if (tiles < g) g = tiles;
     return g < 1 ? 1 : g;
 }
@@ -508,7 +519,7 @@ template <typename T> static size_t red_ws_t(adc_op op, int64_t n) {
     }
     const int items = op == ADC_OP_SOP ? RedItems<T>::pair : RedItems<T>::scalar;
     const int64_t tiles = (n + kRedThreads * items - 1) / (kRedThreads * items);
-    return kWsHeader + (size_t)(simple_grid(tiles) + 1) * 32 + 256;
+    return kWsHeader + (size_t)(simple_grid(tiles, kRedBlocksPerSM) + 1) * 32 + 256;
 }
 
 size_t reduce_ws_bytes(adc_op op, adc_dtype dt, int64_t n) {
@@ -539,10 +550,11 @@ template <class Op, typename T, int ITEMS, class Fin>
 static adc_status launch_simple(const Op &op, const Fin &fin, const T *x, int64_t n, void *ws, cudaStream_t s) {
     constexpr int TILE = kRedThreads * ITEMS;
     const int64_t tiles = (n + TILE - 1) / TILE;
-    const int64_t G = simple_grid(tiles);
+    constexpr int BLOCKS = red_blocks<Op>();
+    const int64_t G = simple_grid(tiles, BLOCKS);
     const int64_t tpb = tiles > 0 ? (tiles + G - 1) / G : 0;
     auto *part = reinterpret_cast<typename Op::State *>(static_cast<char *>(ws) + kWsHeader);
-    k_reduce_simple<Op, Fin, T, ITEMS><<<(unsigned)G, kRedThreads, 0, s>>>(op, fin, x, n, tpb, part,
+    k_reduce_simple<Op, Fin, T, ITEMS, BLOCKS><<<(unsigned)G, kRedThreads, 0, s>>>(op, fin, x, n, tpb, part,
                                                                             counter_slot(ws, 1));
     return check_launch();
 }
