@@ -101,39 +101,51 @@ struct LRank {
 __device__ __forceinline__ void tag_write(int32_t key, bool ok, uint8_t *tag) {
     if (ok) tag[key] = (uint8_t)(threadIdx.x & 31);
 }
-// After a __syncwarp() that follows tag_write(); true if two lanes share a bin.
-__device__ __forceinline__ bool ranks(int32_t key, bool ok, const uint8_t *tag, LRank &r) {
+// After a __syncwarp() that follows tag_write(); the lanes of the fullest bin
+// (1: no two share one), found here once rather than by a vote before every step.
+__device__ __forceinline__ int ranks(int32_t key, bool ok, const uint8_t *tag, LRank &r) {
     const int lane = threadIdx.x & 31;
     unsigned lost = __ballot_sync(0xffffffffu, ok && tag[key] != (uint8_t)lane);
     r = {0, 1};
-    if (lost == 0u) return false;
+    if (lost == 0u) return 1;
+    int steps = 1;
     unsigned peers = 1u << lane;
     if (__popc(lost) <= 4) {
         while (lost) {
             const int32_t k = __shfl_sync(0xffffffffu, key, __ffs(lost) - 1);
             const unsigned same = __ballot_sync(0xffffffffu, ok && key == k);
             if (ok && key == k) peers = same;
+            steps = __popc(same) > steps ? __popc(same) : steps;
             lost &= ~same;
         }
     } else {
         peers = __match_any_sync(0xffffffffu, ok ? key : -1);
         if (!ok) peers = 1u << lane;
+        steps = (int)__reduce_max_sync(0xffffffffu, (unsigned)__popc(peers));
     }
     r.rank = (uint8_t)__popc(peers & ((1u << lane) - 1u));
     r.cnt = (uint8_t)__popc(peers);
-    return true;
+    return steps;
 }
 // One round's updates: upd() runs for every lane with an in-range key, at once
-// when no two share a bin, else in rank order.
-template <class F>
-__device__ __forceinline__ void ranked_update(bool shared, bool ok, int rank, F &&upd) {
-    if (!shared) {
+// when no two share a bin, else in rank order, in as many steps as the fullest
+// bin has lanes.  Two steps are the usual case and stand outside the loop; with
+// one bin there are 32, where a vote before each step was what the walk did
+// (n = 1e7: m = 1 forward 0.195 -> 0.152 ms, vjp 0.443 -> 0.387; m = 400 vjp
+// 0.105 -> 0.095; m = 1000 0.123 -> 0.109).
+template <class F> __device__ __forceinline__ void ranked_update(int steps, bool ok, int rank, F &&upd) {
+    if (steps == 1) {
         if (ok) upd();
-    } else {
-        for (int q = 0; __any_sync(0xffffffffu, ok && rank >= q); ++q) {
-            if (ok && rank == q) upd();
-            __syncwarp();
-        }
+        return;
+    }
+    if (ok && rank == 0) upd();
+    __syncwarp();
+    if (ok && rank == 1) upd();
+    __syncwarp();
+#pragma unroll 1
+    for (int q = 2; q < steps; ++q) {
+        if (ok && rank == q) upd();
+        __syncwarp();
     }
 }
 
@@ -159,16 +171,16 @@ k_linh_fold(const int32_t *__restrict__ keys, const Pair<T> *__restrict__ vals, 
     LRank rk;
     tag_write(k[0], in_range(k[0], m), tag);
     __syncwarp();
-    bool shared = ranks(k[0], in_range(k[0], m), tag, rk);
+    int steps = ranks(k[0], in_range(k[0], m), tag, rk);
 #pragma unroll
     for (int r = 0; r < C::kRounds; ++r) {
         const int32_t key = k[r];
         const Pair<T> x = v[r];
         const int nx = r + 1 < C::kRounds ? r + 1 : r;
         if (r + 1 < C::kRounds) tag_write(k[nx], in_range(k[nx], m), tag);
-        ranked_update(shared, in_range(key, m), rk.rank, [&] { tab[key] = lf(tab[key], x); });
+        ranked_update(steps, in_range(key, m), rk.rank, [&] { tab[key] = lf(tab[key], x); });
         __syncwarp();
-        if (r + 1 < C::kRounds) shared = ranks(k[nx], in_range(k[nx], m), tag, rk);
+        if (r + 1 < C::kRounds) steps = ranks(k[nx], in_range(k[nx], m), tag, rk);
     }
     __syncthreads();
     for (int j = tid; j < m; j += kLThreads) {
@@ -281,10 +293,10 @@ k_linh_vjp(const int32_t *__restrict__ keys, const Pair<T> *__restrict__ vals, c
     // for the backward walk, where the order is reversed
     Pair<T> p[C::kRounds];
     LRank rk[C::kRounds];
-    unsigned shared = 0;  // bit r: lanes of round r share a bin (uniform)
+    uint32_t steps[C::kRounds / 4] = {};  // a byte for each round (uniform)
     tag_write(k[0], in_range(k[0], m), tag);
     __syncwarp();
-    if (ranks(k[0], in_range(k[0], m), tag, rk[0])) shared |= 1u;
+    steps[0] = (uint32_t)ranks(k[0], in_range(k[0], m), tag, rk[0]);
 #pragma unroll
     for (int r = 0; r < C::kRounds; ++r) {
         const int32_t key = k[r];
@@ -292,13 +304,14 @@ k_linh_vjp(const int32_t *__restrict__ keys, const Pair<T> *__restrict__ vals, c
         const int nx = r + 1 < C::kRounds ? r + 1 : r;
         if (r + 1 < C::kRounds) tag_write(k[nx], in_range(k[nx], m), tag);
         Pair<T> pr = lf_id<T>();
-        ranked_update((shared >> r) & 1u, in_range(key, m), rk[r].rank, [&] {
+        ranked_update((int)((steps[r / 4] >> (8 * (r % 4))) & 255u), in_range(key, m), rk[r].rank, [&] {
             pr = tab[key];
             tab[key] = lf(pr, x);
         });
         p[r] = pr;
         __syncwarp();
-        if (r + 1 < C::kRounds && ranks(k[nx], in_range(k[nx], m), tag, rk[nx])) shared |= 1u << nx;
+        if (r + 1 < C::kRounds)
+            steps[nx / 4] |= (uint32_t)ranks(k[nx], in_range(k[nx], m), tag, rk[nx]) << (8 * (nx % 4));
     }
     // backward walk: s_i = product of the c's of i's bin after i in the run
     T sv[C::kRounds];
@@ -307,7 +320,7 @@ k_linh_vjp(const int32_t *__restrict__ keys, const Pair<T> *__restrict__ vals, c
         const int32_t key = k[r];
         const T xc = v[r].c;
         T sr = T(1);
-        ranked_update((shared >> r) & 1u, in_range(key, m), rk[r].cnt - 1 - rk[r].rank, [&] {
+        ranked_update((int)((steps[r / 4] >> (8 * (r % 4))) & 255u), in_range(key, m), rk[r].cnt - 1 - rk[r].rank, [&] {
             sr = qt[key];
             qt[key] = xc * sr;
         });
