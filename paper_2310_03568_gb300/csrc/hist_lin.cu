@@ -196,70 +196,152 @@ k_linh_fold(const int32_t *__restrict__ keys, const Pair<T> *__restrict__ vals, 
 // (the product of the c's after it; the vjp needs no more of the suffix),
 // hist[j] and the bin total A[j], from the columns P[.][j].  The matrices are
 // chunk-major, so that the chunk kernels read and write them in order
-// (bin-major, each of a chunk's 8-byte cells was a sector of its own); a block
+// (bin-major, each of a chunk's 8-byte cells was a sector of its own).  A block
 // takes kColBins bins -- 64 contiguous bytes of a row -- and cuts their columns
-// into kColSegs segments, one thread each: fold the segment, combine the
-// segments through shared memory, walk it again forwards for L and backwards
-// for Rc (both walks read from L2).
+// into kColSegs segments, one thread each: fold the segment, scan the segments
+// (one warp per bin), walk it again forwards for L and backwards for Rc (both
+// walks read from L2).  Bound by the latency of the loads, kColRows rows at a
+// time, so with few bins and many chunks, where the bins alone are a handful of
+// blocks, the rows are split over further blocks too (grid.y), behind a pass
+// that folds each block's rows: col_splits().  n = 1e8, m = 31: four blocks took
+// 0.2 ms of a 0.687 ms forward, now 0.506; m = 100 0.596 -> 0.422; m = 1000 has
+// blocks enough.
 constexpr int kColBins = 8;
 constexpr int kColSegs = kLThreads / kColBins;
+constexpr int kColRows = 8;  // loads in flight
+static_assert(kColSegs == kWarp && kColBins == kLWarps, "a warp scans one bin's segments");
+
+// One thread's segment: rows [c0, c1) of the block's rows [r0, r1), and its fold.
+template <typename T> struct ColSegment {
+    int64_t c0, c1;
+    Pair<T> fold;
+    __device__ ColSegment(const Pair<T> *col, int64_t m, int64_t r0, int64_t r1, int sg, bool live) {
+        int64_t per = (r1 - r0 + kColSegs - 1) / kColSegs;
+        if (per < kColRows) per = kColRows;
+        c0 = r0 + sg * per < r1 ? r0 + sg * per : r1;
+        c1 = c0 + per < r1 ? c0 + per : r1;
+        fold = lf_id<T>();
+        if (!live) return;
+        for (int64_t c = c0; c < c1; c += kColRows) {
+            Pair<T> x[kColRows];
+#pragma unroll
+            for (int u = 0; u < kColRows; ++u) x[u] = c + u < c1 ? col[(c + u) * m] : lf_id<T>();
+#pragma unroll
+            for (int u = 0; u < kColRows; ++u) fold = lf(fold, x[u]);
+        }
+    }
+};
+
+// Inclusive scan of a warp's states in lane order.
+template <typename T> __device__ __forceinline__ Pair<T> lf_warp_scan(Pair<T> v) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 1; o < kWarp; o <<= 1) {
+        const Pair<T> up = shfl_up(v, o);
+        if (lane >= o) v = lf(up, v);
+    }
+    return v;
+}
+
+// F[split][j]: the fold of the split's rows of bin j.
+template <typename T>
+__global__ void __launch_bounds__(kLThreads)
+k_linh_colfold(const Pair<T> *__restrict__ P, const int64_t nc, const int64_t m, const int64_t rows,
+               Pair<T> *__restrict__ F) {
+    __shared__ Pair<T> s_fold[kColBins][kColSegs + 1];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, b = threadIdx.x % kColBins, sg = threadIdx.x / kColBins;
+    const int64_t j0 = (int64_t)blockIdx.x * kColBins, r0 = blockIdx.y * rows, r1 = r0 + rows < nc ? r0 + rows : nc;
+    const ColSegment<T> seg(P + j0 + b, m, r0, r1, sg, j0 + b < m);
+    s_fold[b][sg] = seg.fold;
+    __syncthreads();
+    const Pair<T> all = lf_warp_scan(s_fold[warp][lane]);
+    if (lane == kWarp - 1 && j0 + warp < m) F[blockIdx.y * m + j0 + warp] = all;
+}
 
 template <typename T>
 __global__ void __launch_bounds__(kLThreads)
 k_linh_cols(const Pair<T> *__restrict__ P, const Pair<T> *__restrict__ h0, const int64_t nc, const int64_t m,
-            Pair<T> *__restrict__ L, T *__restrict__ Rc, Pair<T> *__restrict__ hist, Pair<T> *__restrict__ A) {
-    constexpr int U = 8;  // loads in flight
-    __shared__ Pair<T> s_fold[kColSegs][kColBins];
-    const int b = threadIdx.x % kColBins, sg = threadIdx.x / kColBins;
-    const int64_t j = (int64_t)blockIdx.x * kColBins + b;
+            const int64_t rows, const Pair<T> *__restrict__ F, Pair<T> *__restrict__ L, T *__restrict__ Rc,
+            Pair<T> *__restrict__ hist, Pair<T> *__restrict__ A) {
+    __shared__ Pair<T> s_fold[kColBins][kColSegs + 1];  // the segments' folds, then what lies before them
+    __shared__ T s_after[kColBins][kColSegs + 1];       // the product of the c's after them
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, b = threadIdx.x % kColBins, sg = threadIdx.x / kColBins;
+    const int64_t j0 = (int64_t)blockIdx.x * kColBins, j = j0 + b;
     const bool live = j < m;
-    const int64_t per = (nc + kColSegs - 1) / kColSegs;
-    const int64_t c0 = sg * per < nc ? sg * per : nc, c1 = c0 + per < nc ? c0 + per : nc;
+    const int64_t r0 = blockIdx.y * rows, r1 = r0 + rows < nc ? r0 + rows : nc;
     const Pair<T> *col = P + j;
-    Pair<T> f = lf_id<T>();
-    if (live)
-        for (int64_t c = c0; c < c1; c += U) {
-            Pair<T> x[U];
+    const ColSegment<T> seg(col, m, r0, r1, sg, live);
+    s_fold[b][sg] = seg.fold;
+    __syncthreads();
+    {
+        const int64_t jw = j0 + warp;  // the warp's bin
+        // the rows of the other splits: the fold of the earlier ones, the c's of the later ones
+        Pair<T> pre = lf_id<T>();
+        T post = T(1);
+        for (int q0 = 0; q0 < (int)gridDim.y && gridDim.y > 1; q0 += kWarp) {
+            const int q = q0 + lane;
+            const Pair<T> x = q < (int)gridDim.y && jw < m ? F[q * m + jw] : lf_id<T>();
+            const Pair<T> inc = lf_warp_scan(q < (int)blockIdx.y ? x : lf_id<T>());
+            pre = lf(pre, shfl_idx(inc, kWarp - 1));
+            T c = q > (int)blockIdx.y ? x.c : T(1);
 #pragma unroll
-            for (int u = 0; u < U; ++u) x[u] = c + u < c1 ? col[(c + u) * m] : lf_id<T>();
-#pragma unroll
-            for (int u = 0; u < U; ++u) f = lf(f, x[u]);
+            for (int o = 1; o < kWarp; o <<= 1) c *= __shfl_xor_sync(0xffffffffu, c, o);
+            post *= c;
         }
-    s_fold[sg][b] = f;
+        const Pair<T> own = s_fold[warp][lane], inc = lf_warp_scan(own);
+        Pair<T> ex = shfl_up(inc, 1);
+        T suf = own.c;
+#pragma unroll
+        for (int o = 1; o < kWarp; o <<= 1) {
+            const T dn = __shfl_down_sync(0xffffffffu, suf, o);
+            if (lane + o < kWarp) suf = dn * suf;
+        }
+        T after = __shfl_down_sync(0xffffffffu, suf, 1);
+        if (lane == 0) ex = lf_id<T>();
+        if (lane == kWarp - 1) after = T(1);
+        s_fold[warp][lane] = lf(pre, ex);
+        s_after[warp][lane] = post * after;
+        if (lane == kWarp - 1 && blockIdx.y == gridDim.y - 1 && jw < m) {
+            const Pair<T> all = lf(pre, inc);
+            A[jw] = all;
+            hist[jw] = h0 ? lf(h0[jw], all) : all;
+        }
+    }
     __syncthreads();
     if (!live) return;
-    Pair<T> before = lf_id<T>();
-    for (int q = 0; q < sg; ++q) before = lf(before, s_fold[q][b]);
-    T after = T(1);
-    for (int q = kColSegs - 1; q > sg; --q) after = s_fold[q][b].c * after;
-    if (sg == kColSegs - 1) {
-        const Pair<T> all = lf(before, f);
-        A[j] = all;
-        hist[j] = h0 ? lf(h0[j], all) : all;
-    }
-    Pair<T> run = h0 ? lf(h0[j], before) : before;
-    for (int64_t c = c0; c < c1; c += U) {
-        Pair<T> x[U];
+    Pair<T> run = h0 ? lf(h0[j], s_fold[b][sg]) : s_fold[b][sg];
+    T after = s_after[b][sg];
+    for (int64_t c = seg.c0; c < seg.c1; c += kColRows) {
+        Pair<T> x[kColRows];
 #pragma unroll
-        for (int u = 0; u < U; ++u) x[u] = c + u < c1 ? col[(c + u) * m] : lf_id<T>();
+        for (int u = 0; u < kColRows; ++u) x[u] = c + u < seg.c1 ? col[(c + u) * m] : lf_id<T>();
 #pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (c + u < c1) {
+        for (int u = 0; u < kColRows; ++u)
+            if (c + u < seg.c1) {
                 L[(c + u) * m + j] = run;
                 run = lf(run, x[u]);
             }
     }
-    for (int64_t c = c1; c > c0; c -= U) {
-        T x[U];
+    for (int64_t c = seg.c1; c > seg.c0; c -= kColRows) {
+        T x[kColRows];
 #pragma unroll
-        for (int u = 0; u < U; ++u) x[u] = c - 1 - u >= c0 ? col[(c - 1 - u) * m].c : T(1);
+        for (int u = 0; u < kColRows; ++u) x[u] = c - 1 - u >= seg.c0 ? col[(c - 1 - u) * m].c : T(1);
 #pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (c - 1 - u >= c0) {
+        for (int u = 0; u < kColRows; ++u)
+            if (c - 1 - u >= seg.c0) {
                 Rc[(c - 1 - u) * m + j] = after;
                 after = x[u] * after;
             }
     }
+}
+
+// Splits of the rows: so many that the blocks fill the SMs once, each with a
+// full step of every thread's loads at least, and none where the bins alone are
+// a block for every second SM.
+static int64_t col_splits(int64_t nc, int64_t m) {
+    const int64_t blocks = (m + kColBins - 1) / kColBins, want = num_sms() / blocks;
+    const int64_t most = nc / (kColSegs * kColRows);
+    return want < 2 || most < 2 ? 1 : want < most ? want : most;
 }
 
 // ------------------------------------------------------------------- vjp --
@@ -430,9 +512,15 @@ static adc_status linh_fwd_t(int64_t n, int64_t m, const int32_t *keys, const Pa
     if (cudaFuncSetAttribute(k_linh_fold<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return ADC_ERR_CUDA;
     k_linh_fold<T><<<(unsigned)nc, kLThreads, smem, s>>>(keys, vals, n, (int)m, nc, P);
-    k_linh_cols<T><<<(unsigned)((m + kColBins - 1) / kColBins), kLThreads, 0, s>>>(
-        P, h0, nc, m, reinterpret_cast<Pair<T> *>(sv + Lo.L), reinterpret_cast<T *>(sv + Lo.R), hist,
-        reinterpret_cast<Pair<T> *>(sv + Lo.A));
+    const int64_t blocks = (m + kColBins - 1) / kColBins, want = col_splits(nc, m);
+    const int64_t rows = (nc + want - 1) / want, splits = (nc + rows - 1) / rows;
+    const dim3 grid((unsigned)blocks, (unsigned)splits);
+    T *Rc = reinterpret_cast<T *>(sv + Lo.R);
+    // (the upper half of the residuals' Rc is free, and a split has at least two rows)
+    Pair<T> *F = reinterpret_cast<Pair<T> *>(sv + Lo.R + align_up((size_t)m * nc * sizeof(T), 16));
+    if (splits > 1) k_linh_colfold<T><<<grid, kLThreads, 0, s>>>(P, nc, m, rows, F);
+    k_linh_cols<T><<<grid, kLThreads, 0, s>>>(P, h0, nc, m, rows, F, reinterpret_cast<Pair<T> *>(sv + Lo.L), Rc, hist,
+                                              reinterpret_cast<Pair<T> *>(sv + Lo.A));
     return check_launch();
 }
 
