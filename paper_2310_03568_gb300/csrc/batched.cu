@@ -363,18 +363,21 @@ k_b_scan_loss(const adc_instance *__restrict__ desc, const int32_t count, float 
                     }
             }
         }
+        // A thread's bins are summed from zero and what lies before them is added to
+        // each sum: one rounding at the prefix's magnitude per bin, however many bins
+        // a thread has.
         float sum = 0.f;
 #pragma unroll
-        for (int c = 0; c < I; ++c) sum += x[c];
+        for (int c = 0; c < I; ++c) {
+            sum += x[c];
+            x[c] = sum;
+        }
         float total;
         const float inc = block_incl_sum(sum, tmp, &total);
-        float run = carry + __shfl_up_sync(0xffffffffu, inc, 1);
-        if ((threadIdx.x & 31) == 0) run = carry + (threadIdx.x > 0 ? tmp[(threadIdx.x >> 5) - 1] : 0.f);
+        float before = carry + __shfl_up_sync(0xffffffffu, inc, 1);
+        if ((threadIdx.x & 31) == 0) before = carry + (threadIdx.x > 0 ? tmp[(threadIdx.x >> 5) - 1] : 0.f);
 #pragma unroll
-        for (int c = 0; c < I; ++c) {
-            run += x[c];
-            x[c] = j0 + c < d.m ? run : 0.f;
-        }
+        for (int c = 0; c < I; ++c) x[c] = j0 + c < d.m ? before + x[c] : 0.f;
         add_group(acc, x);
         if (whole) {
 #pragma unroll
