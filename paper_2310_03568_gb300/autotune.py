@@ -1,22 +1,25 @@
 """Autotuner for the launch parameters libadcomb exposes.
 
 * batched hist -> scan -> sum: work-item size (``chunk``), shared-memory
-  table size (``smem_bins``) and elements per thread and step (``items``) of
-  the persistent histogram launch;
+  table size (``smem_bins``, 0 for the library's own) and elements per thread
+  and step (``items``) of the persistent histogram launch;
 * reduce_by_index (single call): the forward strategy -- per-thread tables,
   per-warp copies, one block-wide table, global atomics, or partitioning by bin
   range into shared-memory-sized buckets
   (``adc_debug_force_hist_strategy``; the library validates that the table fits);
-* scan (single call): items per thread and tile shape -- 64 contiguous bytes
-  per thread and tile, or 16 bytes (a warp's load then covers 512 contiguous
-  bytes), each with the range-partitioned engine at several tiles per range;
-  the per-tile look-back engine; and one tile per block staged in shared
-  memory by bulk copies (``adc_debug_set_scan_engine``,
+* scan (single call): the library's own choice (the streaming engine from 3 MB
+  per input array on, the per-tile engine below); items per thread and tile
+  shape -- 64 contiguous bytes per thread and tile, or 16 bytes (a warp's load
+  then covers 512 contiguous bytes), each with the range-partitioned engine at
+  several tiles per range; the per-tile look-back engine; and one tile per block
+  staged in shared memory by bulk copies (``adc_debug_set_scan_engine``,
   ``adc_debug_set_scan_range_tiles``).
 
 Each candidate is timed with CUDA events on the real inputs (warm-up, then the
 mean of a few runs); the winner is cached in a JSON file keyed by the shape
-bucket, so later calls with a similar shape reuse it without measuring.
+bucket, so later calls with a similar shape reuse it without measuring.  The
+key also holds a digest of the library's sources: a number measured on other
+kernels says nothing about these, and would pin their best choice for good.
 Cache file: ``$ADC_AUTOTUNE_CACHE`` or ``~/.cache/adcomb_autotune.json``.
 """
 from __future__ import annotations
@@ -29,18 +32,20 @@ import threading
 import torch
 
 from . import adcomb
+from .build import source_digest
 
 _lock = threading.Lock()
 _cache = None
+_digest = None
 
 BATCHED_CHUNKS = (1 << 14, 1 << 16, 1 << 18)
-BATCHED_SMEM_BINS = (4096, 8192, 16384)
+BATCHED_SMEM_BINS = (0, 4096, 8192, 16384)  # 0: the library's default
 BATCHED_ITEMS = (1, 4, 8)
 HIST_STRATEGIES = (3, 0, 1, 2, 4, 5, 6, 7)  # per-thread, per-warp, per-block, global, partitioned, split,
                                           # cluster, two passes
-# scan candidates (engine, tiles per range): 64-byte items with the automatic
-# choice and with ranges of 16 / 32 tiles; the per-tile engine; 16-byte items
-# with the default and 32-tile ranges; one TMA-staged tile per block
+# scan candidates (engine, tiles per range): the automatic choice; 64-byte items
+# in ranges of 16 / 32 tiles; the per-tile engine; 16-byte items with the default
+# and 32-tile ranges; one TMA-staged tile per block
 SCAN_CANDIDATES = ((0, 0), (2, 16), (2, 32), (1, 0), (5, 0), (5, 32), (4, 0))
 
 
@@ -76,6 +81,14 @@ def _bucket(x):
     return int(round(math.log2(max(int(x), 1))))
 
 
+def _kernels():
+    """The device and the kernels that a measurement belongs to."""
+    global _digest
+    if _digest is None:
+        _digest = source_digest()
+    return f"{torch.cuda.get_device_name()}|{_digest}"
+
+
 def _time(fn, reps=3):
     fn()
     torch.cuda.synchronize()
@@ -89,8 +102,7 @@ def _time(fn, reps=3):
 
 
 def batched_key(desc):
-    dev = torch.cuda.get_device_name()
-    return (f"batched|{dev}|count={_bucket(len(desc))}|n={_bucket(desc['n'].sum())}|"
+    return (f"batched|{_kernels()}|count={_bucket(len(desc))}|n={_bucket(desc['n'].sum())}|"
             f"mmean={_bucket(desc['m'].mean())}")
 
 
@@ -129,7 +141,7 @@ def tune_batched(problem, force=False):
 
 
 def hist_key(op, dtype, n, m):
-    return f"hist|{torch.cuda.get_device_name()}|{op}|{dtype}|n={_bucket(n)}|m={_bucket(m)}"
+    return f"hist|{_kernels()}|{op}|{dtype}|n={_bucket(n)}|m={_bucket(m)}"
 
 
 def tune_hist(op, m, keys, vals, force=False):
@@ -157,7 +169,7 @@ def tune_hist(op, m, keys, vals, force=False):
 
 
 def scan_key(op, dtype, n):
-    return f"scan|{torch.cuda.get_device_name()}|{op}|{dtype}|n={_bucket(n)}"
+    return f"scan|{_kernels()}|{op}|{dtype}|n={_bucket(n)}"
 
 
 def tune_scan(op, x, force=False):
