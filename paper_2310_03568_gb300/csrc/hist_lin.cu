@@ -154,7 +154,7 @@ template <class F> __device__ __forceinline__ void ranked_update(int steps, bool
 template <typename T>
 __global__ void __launch_bounds__(kLThreads)
 k_linh_fold(const int32_t *__restrict__ keys, const Pair<T> *__restrict__ vals, const int64_t n, const int m,
-            const int64_t nc, Pair<T> *__restrict__ P) {
+            Pair<T> *__restrict__ P) {
     using C = LChunk<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Pair<T> *s_tab = reinterpret_cast<Pair<T> *>(smem_raw);              // [kLWarps][m]
@@ -348,8 +348,8 @@ static int64_t col_splits(int64_t nc, int64_t m) {
 template <typename T>
 __global__ void __launch_bounds__(kLThreads, 2)
 k_linh_vjp(const int32_t *__restrict__ keys, const Pair<T> *__restrict__ vals, const int64_t n, const int m,
-           const int64_t nc, const Pair<T> *__restrict__ L, const T *__restrict__ Rc,
-           const Pair<T> *__restrict__ hb, Pair<T> *__restrict__ vbar, const int accumulate) {
+           const Pair<T> *__restrict__ L, const T *__restrict__ Rc, const Pair<T> *__restrict__ hb,
+           Pair<T> *__restrict__ vbar, const int accumulate) {
     using C = LChunk<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Pair<T> *s_tab = reinterpret_cast<Pair<T> *>(smem_raw);  // [kLWarps][m]: folds, then (before . g, after.c)
@@ -511,7 +511,7 @@ static adc_status linh_fwd_t(int64_t n, int64_t m, const int32_t *keys, const Pa
     const size_t smem = fold_smem<T>(m);
     if (cudaFuncSetAttribute(k_linh_fold<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return ADC_ERR_CUDA;
-    k_linh_fold<T><<<(unsigned)nc, kLThreads, smem, s>>>(keys, vals, n, (int)m, nc, P);
+    k_linh_fold<T><<<(unsigned)nc, kLThreads, smem, s>>>(keys, vals, n, (int)m, P);
     const int64_t blocks = (m + kColBins - 1) / kColBins, want = col_splits(nc, m);
     const int64_t rows = (nc + want - 1) / want, splits = (nc + rows - 1) / rows;
     const dim3 grid((unsigned)blocks, (unsigned)splits);
@@ -537,7 +537,7 @@ static adc_status linh_vjp_t(int64_t n, int64_t m, const int32_t *keys, const Pa
         const size_t smem = vjp_smem<T>(m);
         if (cudaFuncSetAttribute(k_linh_vjp<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
             return ADC_ERR_CUDA;
-        k_linh_vjp<T><<<(unsigned)nc, kLThreads, smem, s>>>(keys, vals, n, (int)m, nc, L, R, hb, vb, acc);
+        k_linh_vjp<T><<<(unsigned)nc, kLThreads, smem, s>>>(keys, vals, n, (int)m, L, R, hb, vb, acc);
     }
     if (h0b) {
         const int64_t g = (m + 255) / 256;

@@ -543,13 +543,6 @@ template <typename T, int ITEMS> struct VjpMM2 {
         fetch_next_sm(sm[1], lo, c0, n, r.x, mat_eye<T>());
         fetch_prev_sm(sm[2], lo, c0, n, r.y, mat_eye<T>());
     }
-    static constexpr int kWalk = 1;
-    using Scalar = T;
-    __device__ Elem *dst() const { return xbar; }
-    __device__ bool accumulating() const { return accumulate != 0; }
-    __device__ Mat2<T> pad(int s) const { return s == 0 ? mat_zero<T>() : mat_eye<T>(); }
-    __device__ State item(const Mat2<T> &yb, const Mat2<T> &xn) const { return {yb, mat_t(xn)}; }
-    __device__ Mat2<T> out(const State &run, const Mat2<T> &yp) const { return mat_mul(mat_t(yp), run.v); }
     __device__ void build(int64_t c0, int64_t n, const Raw &r, State (&st)[ITEMS], Aux &aux) const {
 #pragma unroll
         for (int k = 0; k < ITEMS; ++k) {
@@ -863,10 +856,16 @@ template <class Op> struct StreamPick {
     static constexpr bool kSplit = !one && f32;
 };
 // From 3 MB per input array on (about one 32 KB tile for every second SM) the
-// streaming engine is the faster one at every size measured: + n = 1e6 0.0139 ->
-// 0.0133 ms, 2e6 0.0214 -> 0.0157, 1e7 0.0352 -> 0.0235, 1e8 0.215 -> 0.136;
-// below, both are bound by their launches and the per-tile engine has the
-// smaller blocks.  A tuned range length asks for the range engine.
+// streaming engine is the faster one for every operator, direction and type, at
+// 3, 4, 6, 12, 24 and 48 MB.  At 3 MB, us, per-tile engine -> streaming:
+//           +              *              max            lin            sumOfProd
+//   fp32    14.3 -> 10.2   14.9 -> 10.3   14.2 -> 10.8   12.3 ->  9.0   12.7 ->  8.6
+//   vjp     14.4 -> 10.2   14.3 -> 12.2   14.5 -> 11.5   16.4 -> 12.6   22.8 -> 12.6
+//   fp64    16.1 -> 13.1   16.0 -> 13.1   17.0 -> 13.6   17.6 -> 14.3   21.2 -> 16.9
+//   vjp     16.2 -> 13.1   28.0 -> 17.9   28.7 -> 22.3   35.4 -> 19.7   40.6 -> 22.0
+// (2x2 forward fp32 13.9 -> 9.2).  Below, both are bound by their launches and
+// the per-tile engine has the smaller blocks.  A tuned range length asks for the
+// range engine.
 constexpr int64_t kStreamMinBytes = 3 << 20;
 
 template <class Op, int ITEMS, bool REVERSE>

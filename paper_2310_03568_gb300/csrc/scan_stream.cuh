@@ -71,7 +71,8 @@ __device__ __forceinline__ void mbar_arrive(unsigned long long *bar) {
 
 template <class Op, int NWC, int RB, int STAGES> struct StreamShape {
     using E = typename Op::Elem;
-    static constexpr int U = sizeof(E) > 16 ? (int)sizeof(E) : 16;  // bytes loaded at once by a row walk
+    static_assert(sizeof(E) <= 16 && (RB == 64 || RB == 128), "a unit holds whole elements; row_swizzle()");
+    static constexpr int U = 16;                                    // bytes loaded at once by a row walk
     static constexpr int NPU = U / (int)sizeof(E);                  // elements in them
     static constexpr int UR = RB / U;                               // and how many to a row
     static constexpr int C = RB / 16;                               // 16-byte chunks per row
@@ -87,7 +88,7 @@ template <class Op, int NWC, int RB, int STAGES> struct StreamShape {
 };
 
 template <int RB> __device__ __forceinline__ int row_swizzle(int row) {
-    return RB == 128 ? (row & 7) : RB == 64 ? ((row >> 1) & 3) : ((row >> 2) & 1);
+    return RB == 128 ? (row & 7) : ((row >> 1) & 3);
 }
 
 // One warp's segment of one stream in a stage.
@@ -98,19 +99,13 @@ template <class Sh, int RB> struct Segment {
         return p + row * RB + ((c ^ row_swizzle<RB>(row)) << 4);
     }
     __device__ __forceinline__ void load(int row, int u, E (&v)[Sh::NPU]) const {
-#pragma unroll
-        for (int w = 0; w < Sh::U / 16; ++w) {
-            const uint4 t = *reinterpret_cast<const uint4 *>(chunk(row, u * (Sh::U / 16) + w));
-            memcpy(reinterpret_cast<unsigned char *>(v) + 16 * w, &t, 16);
-        }
+        const uint4 t = *reinterpret_cast<const uint4 *>(chunk(row, u));
+        memcpy(v, &t, 16);
     }
     __device__ __forceinline__ void store(int row, int u, const E (&v)[Sh::NPU]) const {
-#pragma unroll
-        for (int w = 0; w < Sh::U / 16; ++w) {
-            uint4 t;
-            memcpy(&t, reinterpret_cast<const unsigned char *>(v) + 16 * w, 16);
-            *reinterpret_cast<uint4 *>(chunk(row, u * (Sh::U / 16) + w)) = t;
-        }
+        uint4 t;
+        memcpy(&t, v, 16);
+        *reinterpret_cast<uint4 *>(chunk(row, u)) = t;
     }
     // first element of the row after `row`, last element of the row before it
     __device__ __forceinline__ E after(int row) const {
@@ -129,26 +124,21 @@ template <class Sh, int RB> struct Segment {
 
 // Copies the 16 bytes at byte offset b of an array of nb bytes into shared
 // memory: asynchronously when they lie inside it, else element by element
-// with `pad` outside.  `part`: which 16 bytes of a larger element they are.
+// with `pad` outside.
 template <typename E>
-__device__ __forceinline__ void copy16(unsigned char *dst, const E *src, int64_t b, int64_t nb, const E &pad,
-                                       int part) {
+__device__ __forceinline__ void copy16(unsigned char *dst, const E *src, int64_t b, int64_t nb, const E &pad) {
     if (b >= 0 && b + 16 <= nb) {
         cp_async16(dst, reinterpret_cast<const unsigned char *>(src) + b);
         return;
     }
-    uint4 t;
-    if constexpr (sizeof(E) <= 16) {
-        E v[16 / sizeof(E)];
+    E v[16 / sizeof(E)];
 #pragma unroll
-        for (int k = 0; k < (int)(16 / sizeof(E)); ++k) {
-            const int64_t at = b + k * (int64_t)sizeof(E);
-            v[k] = (at >= 0 && at < nb) ? src[at / (int64_t)sizeof(E)] : pad;
-        }
-        memcpy(&t, v, 16);
-    } else {
-        memcpy(&t, reinterpret_cast<const unsigned char *>(&pad) + 16 * part, 16);
+    for (int k = 0; k < (int)(16 / sizeof(E)); ++k) {
+        const int64_t at = b + k * (int64_t)sizeof(E);
+        v[k] = (at >= 0 && at < nb) ? src[at / (int64_t)sizeof(E)] : pad;
     }
+    uint4 t;
+    memcpy(&t, v, 16);
     *reinterpret_cast<uint4 *>(dst) = t;
 }
 
@@ -269,7 +259,7 @@ __device__ __forceinline__ bool stream_lookback(const Op &op, const unsigned lon
     using S = typename Op::State;
     constexpr int K = Tagged<S>::K;
     constexpr int Q = 5;  // 160 tiles: one per SM, so one step as a rule
-    constexpr bool kLaneMajor = K > 4 || sizeof(typename Op::Scalar) == 8;
+    constexpr bool kLaneMajor = sizeof(typename Op::Scalar) == 8;
     const unsigned lane = threadIdx.x & 31;
     for (unsigned base = from; base < to; base += 32 * Q) {
         unsigned long long w[Q][K];
@@ -490,16 +480,12 @@ k_scan_stream(const Op op, const int64_t n, const int64_t num_tiles, unsigned lo
                     const E pad = op.pad(s);
                     for (int j = 0; j < Sh::C; ++j) {
                         const int q = j * 32 + lane;
-                        copy16(d.chunk(q / Sh::C, q % Sh::C), src, b0 + q * 16, nb, pad, q % (Sh::U / 16));
+                        copy16(d.chunk(q / Sh::C, q % Sh::C), src, b0 + q * 16, nb, pad);
                     }
                 }
                 if constexpr (Op::kWalk != 0) {  // one unit after the segment, one before it
-                    if (s > 0 && lane < 2 * (Sh::U / 16)) {
-                        const int part = lane % (Sh::U / 16);
-                        const bool prev = lane >= Sh::U / 16;
-                        const int64_t b = (prev ? b0 - Sh::U : b0 + Sh::SEG) + 16 * part;
-                        copy16(d.p + Sh::SEG + 16 * lane, src, b, nb, op.pad(s), part);
-                    }
+                    if (s > 0 && lane < 2)
+                        copy16(d.p + Sh::SEG + 16 * lane, src, lane ? b0 - Sh::U : b0 + Sh::SEG, nb, op.pad(s));
                 }
             }
         }
