@@ -109,7 +109,11 @@ k_sort_scatter(const int32_t *__restrict__ keys, const int32_t *__restrict__ per
     extern __shared__ int32_t s_w[];  // [8 warps][buckets]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int NW = kSortThreads / kWarp;
-    if (__ldcg(err) != 0u) {
+    __shared__ unsigned s_err;
+    if (threadIdx.x == 0) s_err = __ldcg(err);
+    for (int j = threadIdx.x; j < NW * P.buckets; j += kSortThreads) s_w[j] = 0;
+    __syncthreads();
+    if (s_err != 0u) {
         for (int r = 0; r < kSortRounds; ++r) {
             const int64_t i = (int64_t)blockIdx.x * kSortTile + (int64_t)r * kSortThreads + threadIdx.x;
             if (i >= n) break;
@@ -119,8 +123,6 @@ k_sort_scatter(const int32_t *__restrict__ keys, const int32_t *__restrict__ per
         }
         return;
     }
-    for (int j = threadIdx.x; j < NW * P.buckets; j += kSortThreads) s_w[j] = 0;
-    __syncthreads();
     int32_t *wc = s_w + warp * P.buckets;
     const int64_t base = (int64_t)blockIdx.x * kSortTile + (int64_t)warp * (kSortTile / NW);
     const unsigned lt = (1u << lane) - 1u;
