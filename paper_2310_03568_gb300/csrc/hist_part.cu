@@ -423,7 +423,7 @@ k_part_scatter(const int32_t *__restrict__ keys, const T *__restrict__ vals, con
     }
 }
 
-// 3 (fp32). The same counting sort with the chunk staged in shared memory:
+// 2 (fp32). The same counting sort with the chunk staged in shared memory:
 // persistent blocks, two per SM, each taking chunks b, b + G, ...; a whole
 // chunk's keys and values arrive by two bulk copies, and while one block waits
 // for its copy, ranks, scans or stores, the other one works (one block per SM
@@ -441,9 +441,9 @@ inline size_t scat_smem(int B) { return (size_t)kPartChunk * (4 + 4 + 2) + (size
 template <int MODE>
 __global__ void __launch_bounds__(kScatThreads, 2)
 k_part_scatter_tma(const int32_t *__restrict__ keys, const float *__restrict__ vals, const int64_t n, const int64_t m,
-                   const BucketDiv bdiv, const int B, const int64_t nchunks, int32_t *__restrict__ cursor,
-                   uint16_t *__restrict__ obin, typename PartTraits<float, MODE>::V *__restrict__ oval,
-                   const DevCtl ctl) {
+                   const BucketDiv bdiv, const int B, const int64_t nchunks, int32_t *__restrict__ start,
+                   int32_t *__restrict__ cursor, uint16_t *__restrict__ obin,
+                   typename PartTraits<float, MODE>::V *__restrict__ oval, const DevCtl ctl) {
     using Tr = PartTraits<float, MODE>;
     constexpr int NW = kScatThreads / kWarp;
     constexpr int PER = kPartMaxBuckets / kScatThreads;  // buckets per thread in the local scan
@@ -479,7 +479,12 @@ k_part_scatter_tma(const int32_t *__restrict__ keys, const float *__restrict__ v
         const int len = (int)((n - e0) < kPartChunk ? (n - e0) : kPartChunk);
         if (whole(c)) {
             const bool ok = mbar_wait_bounded(&s_bar, used & 1u, ctl.spin_limit);
-            if (!__syncthreads_and(ok)) {  // report, let the copy land, leave: the table pass touches nothing
+            if (!__syncthreads_and(ok)) {
+                // Report, let the copy land, leave.  This block's share of the runs stays
+                // unwritten, and what lies there is neither a bin nor an element: all runs
+                // are made empty for the table pass (a check of the error word there cost
+                // every call 0.5 to 1 us).
+                for (int b = tid; b <= B; b += kScatThreads) start[b] = 0;
                 if (tid == 0) {
                     set_error(ctl.err, kErrTimeout);
                     if (c != ctl.stall_tile) mbar_drain(&s_bar, used & 1u);
@@ -573,10 +578,8 @@ k_part_scatter_tma(const int32_t *__restrict__ keys, const float *__restrict__ v
 }
 
 // 3. One block per bucket: the bucket's W bins in shared memory, its run of
-// (bin, payload) streamed in, the bins written out.  A scatter block that gave
-// up on its copy left its share of the runs unwritten, and what lies there is
-// neither a bin nor an element: with a timeout recorded, no element is touched
-// and every bin comes out empty.
+// (bin, payload) streamed in, the bins written out.  After a timeout in the
+// scatter every run is empty, and so is every bin.
 template <typename T, int MODE>
 __global__ void __launch_bounds__(kPartTableThreads)
 k_part_table(const uint16_t *__restrict__ obin, const typename PartTraits<T, MODE>::V *__restrict__ oval,
@@ -590,7 +593,7 @@ k_part_table(const uint16_t *__restrict__ obin, const typename PartTraits<T, MOD
     for (int t = threadIdx.x; t < w; t += kPartTableThreads) Tr::init(smem_raw, (int)W, t);
     __syncthreads();
     const int64_t start = bucket[blockIdx.x];
-    const int64_t end = (__ldcg(err) & kErrTimeout) ? start : bucket[blockIdx.x + 1];
+    const int64_t end = bucket[blockIdx.x + 1];
     constexpr int U = 8;
     for (int64_t g0 = start; g0 < end; g0 += (int64_t)U * kPartTableThreads) {
         int32_t u[U];
@@ -714,7 +717,7 @@ static adc_status part_run(int64_t n, int64_t m, const int32_t *keys, const T *v
         if (!smem_attr(k_part_scatter_tma<MODE>, sm_tma)) return ADC_ERR_CUDA;
         const int64_t two = (int64_t)num_sms() * 2;
         k_part_scatter_tma<MODE><<<(unsigned)(nc < two ? nc : two), kScatThreads, sm_tma, s>>>(
-            keys, vals, n, m, bdiv, P.B, nc, cursor, obin, oval, make_ctl(ws, kPartSlot));
+            keys, vals, n, m, bdiv, P.B, nc, start, cursor, obin, oval, make_ctl(ws, kPartSlot));
     } else {
         const size_t sm_scatter = (size_t)kPartChunk * (sizeof(V) + 4) + (size_t)P.B * 8;
         if (!smem_attr(k_part_scatter<T, MODE>, sm_scatter)) return ADC_ERR_CUDA;
