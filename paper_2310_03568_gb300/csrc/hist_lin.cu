@@ -30,8 +30,8 @@
 // latency of the walks' shared-memory steps, at 16 to 24 warps per SM (the
 // tables fill the shared memory).  n = 1e7, m = 1000, fp32: fold 0.074 -> 0.049
 // ms (ranks found by ballots a round ahead instead of a match in the update's
-// way), columns 0.037 -> 0.029 ms and vjp 0.189 -> 0.118 ms (ranks reused
-// backwards, chunk-major matrices).
+// way), columns 0.037 -> 0.029 ms and vjp 0.189 -> 0.109 ms (ranks reused
+// backwards, chunk-major matrices, no votes in the walks).
 #include "common.cuh"
 #include "hist_common.cuh"
 #include "internal.h"
@@ -131,8 +131,10 @@ __device__ __forceinline__ int ranks(int32_t key, bool ok, const uint8_t *tag, L
 // when no two share a bin, else in rank order, in as many steps as the fullest
 // bin has lanes.  Two steps are the usual case and stand outside the loop; with
 // one bin there are 32, where a vote before each step was what the walk did
-// (n = 1e7: m = 1 forward 0.195 -> 0.152 ms, vjp 0.443 -> 0.387; m = 400 vjp
-// 0.105 -> 0.095; m = 1000 0.123 -> 0.109).
+// (n = 1e7: m = 1 forward 0.195 -> 0.134 ms, vjp 0.442 -> 0.310; m = 400 vjp
+// 0.105 -> 0.096; m = 1000 0.122 -> 0.111).  The loop is unrolled by two: by four,
+// 32 copies of it in the vjp are too much code (m = 31 to 1000 5% to 9% slower),
+// and rolled, m = 1 takes 0.152 and 0.386 ms.
 template <class F> __device__ __forceinline__ void ranked_update(int steps, bool ok, int rank, F &&upd) {
     if (steps == 1) {
         if (ok) upd();
@@ -142,7 +144,7 @@ template <class F> __device__ __forceinline__ void ranked_update(int steps, bool
     __syncwarp();
     if (ok && rank == 1) upd();
     __syncwarp();
-#pragma unroll 1
+#pragma unroll 2
     for (int q = 2; q < steps; ++q) {
         if (ok && rank == q) upd();
         __syncwarp();
