@@ -41,8 +41,8 @@ WORKLOAD = ("reduce_by_index specialisations fp32: n=50M uniform int32 bins, m i
 # scaled to n by the parts that grow with n, plus the m-sized outputs (the
 # partitioned-histogram kernels' capture): the roofline's `traffic` for the
 # dominant call, when it is one of these.
-TRAFFIC_PER_ELEM = {("fwd", "mul", 10_000_000): (22.1, 120e6), ("fwd", "min", 10_000_000): (29.7, 80e6),
-                    ("fwd", "max", 10_000_000): (29.7, 80e6)}
+TRAFFIC_PER_ELEM = {("fwd", "mul", 10_000_000): (21.7, 120e6), ("fwd", "min", 10_000_000): (29.3, 80e6),
+                    ("fwd", "max", 10_000_000): (29.3, 80e6)}
 
 
 def launches(phase, op, m, n):

@@ -195,7 +195,7 @@ adc_status adc_scan_fwd_noalloc(adc_op op, adc_dtype dtype, int64_t n, const voi
  *           SOP -- unused (the vjp reads hist)
  *           LIN -- for m <= 2047 (fp32) / 1023 (fp64): per (bin, input chunk) the exclusive
  *                   prefix and suffix of the bin's fold across chunks, and
- *                   the bin totals (the chunk-local stable sort is redone in
+ *                   the bin totals (the walks over the chunks are redone in
  *                   the vjp); for larger m: the stable sort permutation, the
  *                   sorted keys and the sorted values (general rule, Fig. 4)
  *   ops: ADD, MUL, MIN, MAX, LIN, SOP (LIN is not commutative: the fold follows

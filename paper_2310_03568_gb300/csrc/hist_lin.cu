@@ -30,7 +30,7 @@
 // latency of the walks' shared-memory steps, at 16 to 24 warps per SM (the
 // tables fill the shared memory).  n = 1e7, m = 1000, fp32: fold 0.074 -> 0.049
 // ms (ranks found by ballots a round ahead instead of a match in the update's
-// way), columns 0.037 -> 0.029 ms and vjp 0.189 -> 0.109 ms (ranks reused
+// way), columns 0.037 -> 0.029 ms and vjp 0.189 -> 0.111 ms (ranks reused
 // backwards, chunk-major matrices, no votes in the walks).
 #include "common.cuh"
 #include "hist_common.cuh"
@@ -205,9 +205,9 @@ k_linh_fold(const int32_t *__restrict__ keys, const Pair<T> *__restrict__ vals, 
 // walks read from L2).  Bound by the latency of the loads, kColRows rows at a
 // time, so with few bins and many chunks, where the bins alone are a handful of
 // blocks, the rows are split over further blocks too (grid.y), behind a pass
-// that folds each block's rows: col_splits().  n = 1e8, m = 31: four blocks took
-// 0.2 ms of a 0.687 ms forward, now 0.506; m = 100 0.596 -> 0.422; m = 1000 has
-// blocks enough.
+// that folds each block's rows: col_splits().  Forward at n = 1e8: m = 4 0.838 ->
+// 0.529 ms, m = 31 0.690 -> 0.512, m = 100 0.598 -> 0.404 (together with the
+// walks' counted steps); m = 1000 has blocks enough.
 constexpr int kColBins = 8;
 constexpr int kColSegs = kLThreads / kColBins;
 constexpr int kColRows = 8;  // loads in flight
